@@ -185,8 +185,8 @@ NLC_API nlc_status nlc_set_graph(nlc_ctx* ctx, int32_t steps);
  * between the lb and Beris-Edwards phases of each step; the results equal
  * the two-kernel form bit for bit.  Combines with nlc_set_graph (a graph
  * then holds the cooperative launches).  0 (default): two kernel launches
- * per step.  The MRT collision and devices without cooperative launch keep
- * the two-kernel form.  Errors: NLC_EINVAL (steps < 0). */
+ * per step.  The MRT collision, float64 arithmetic (NLC_FP64, NLC_FP32_QF64)
+ * and devices without cooperative launch keep the form of separate kernels.  Errors: NLC_EINVAL (steps < 0). */
 NLC_API nlc_status nlc_set_persistent(nlc_ctx* ctx, int32_t steps);
 
 /* Finite-difference stencils of the context (every lattice).

@@ -15,6 +15,7 @@
 #include "engine.h"
 #include "nvtx_range.h"
 #include "obs_finish.h"
+#include "step_cell.cuh"
 #include "step_fused.cuh"
 #include "step_unfused.cuh"
 
@@ -85,6 +86,7 @@ struct InstHost {
   Field<T> u;
   int tz = 1;
   T* mrt = nullptr;  // MRT coefficients s_k / |v_k|^2 on the device, or nullptr (BGK)
+  std::vector<double> mrt_coef;  // the same in float64
   // lazily allocated: unfused schedule, read-back staging, checkpoints
   T* pi = nullptr;
   Field<T> qp;
@@ -132,6 +134,8 @@ class Engine final : public EngineBase {
  public:
   static constexpr int Q = Lat::Q;
   static constexpr int DIM = Lat::DIM;
+  // float64 arithmetic: the fused schedule runs the kernels of step_cell.cuh
+  static constexpr bool kCell = std::is_same<T, double>::value;
 
   explicit Engine(const EngineArgs& a) : args_(a) {}
 
@@ -285,7 +289,11 @@ class Engine final : public EngineBase {
       cudaMemcpyAsync(qsave[i], I.q[cur0].base, qb, cudaMemcpyDeviceToDevice, st);
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    nlc_status s = NLC_OK;
+    nlc_status s = ensure_cells();
+    if (s) {
+      release();
+      return s;
+    }
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
       err = "nlc_autotune: cudaEventCreate failed";
       s = NLC_ECUDA;
@@ -382,13 +390,15 @@ class Engine final : public EngineBase {
       if (!I.mrt && (s = alloc(&I.mrt, (size_t)Q))) return s;
       constexpr MomentBasis<Lat> B = make_moment_basis<Lat>();
       T a[Q];
-      for (int k = 0; k < Q; k++) a[k] = (T)(rates[k] / B.n2[k]);
+      I.mrt_coef.resize(Q);
+      for (int k = 0; k < Q; k++) a[k] = (T)(I.mrt_coef[k] = rates[k] / B.n2[k]);
       NLC_CK(cudaMemcpyAsync(I.mrt, a, sizeof(a), cudaMemcpyHostToDevice, st));
     }
     const T* ptr = rates ? I.mrt : nullptr;
     NLC_CK(cudaMemcpyAsync(&insts_dev_[i].mrt, &ptr, sizeof(ptr), cudaMemcpyHostToDevice, st));
     NLC_CK(cudaStreamSynchronize(st));
     mrt_on_[i] = rates != nullptr;
+    cells_stale_ = true;
     any_mrt_ = false;
     for (bool b : mrt_on_) any_mrt_ = any_mrt_ || b;
     drop_graphs();
@@ -410,7 +420,10 @@ class Engine final : public EngineBase {
 
   // stencils of every lattice: standard (false) or isotropic (true)
   nlc_status set_stencil(bool iso) override {
-    if (iso != iso_) drop_graphs();
+    if (iso != iso_) {
+      drop_graphs();
+      cells_stale_ = true;
+    }
     iso_ = iso;
     return NLC_OK;
   }
@@ -422,6 +435,14 @@ class Engine final : public EngineBase {
     // the device descriptor holds the parameters: update it in place
     NLC_CK(cudaMemcpyAsync(&insts_dev_[i].p, &I.p, sizeof(Par<T>), cudaMemcpyHostToDevice,
                            args_.stream));
+    if constexpr (kCell) {
+      if (cells_dev_ && !cells_stale_) {
+        const CellPar c = make_cell_par<Lat>(I.p, iso_);
+        NLC_CK(cudaMemcpyAsync(&cells_dev_[i].c, &c, sizeof(c), cudaMemcpyHostToDevice,
+                               args_.stream));
+        NLC_CK(cudaStreamSynchronize(args_.stream));
+      }
+    }
     NLC_CK(cudaStreamSynchronize(args_.stream));
     return NLC_OK;
   }
@@ -442,8 +463,9 @@ class Engine final : public EngineBase {
             "unfused schedule";
       return NLC_EUNSUPPORTED;
     }
-    // the persistent kernel's occupancy and counters are set up here, not
-    // inside a stream capture (no allocation may happen there)
+    // workspaces, the persistent kernel's occupancy and counters are set up
+    // here, not inside a stream capture (no allocation may happen there)
+    if ((s = ensure_cells())) return s;
     if (persistent_steps > 0 && !any_mrt_) {
       int grid;
       if ((s = persist_grid(&grid))) return s;
@@ -479,8 +501,15 @@ class Engine final : public EngineBase {
     return NLC_OK;
   }
 
-  // blocks of the persistent kernel (0: not available on this device)
+  // blocks of the persistent kernel (0: not available on this device, or
+  // float64 arithmetic, whose steps run as the kernels of step_cell.cuh)
   nlc_status persist_grid(int* grid) {
+    *grid = 0;
+    if constexpr (!kCell) return persist_grid_f32(grid);
+    return NLC_OK;
+  }
+
+  nlc_status persist_grid_f32(int* grid) {
     const int v = (iso_ ? 2 : 0) + (ix32_ ? 1 : 0);
     if (pgrid_max_[v] < 0)
       pgrid_max_[v] = persistent_grid_max<Lat, T, G>(iso_, ix32_);
@@ -494,6 +523,11 @@ class Engine final : public EngineBase {
 
   // m steps of every lattice in one cooperative launch
   nlc_status step_persistent(cudaStream_t st, int m, int grid) {
+    if constexpr (kCell) return NLC_EUNSUPPORTED;  // persist_grid gives 0
+    else return step_persistent_f32(st, m, grid);
+  }
+
+  nlc_status step_persistent_f32(cudaStream_t st, int m, int grid) {
     NLC_CK(cudaMemsetAsync(pbar_, 0, sizeof(GridBarrier), st));
     const int e0 = mark();
     PersistArgs pa{pbar_, wait_ns};
@@ -794,8 +828,9 @@ class Engine final : public EngineBase {
     const Dims& d = I.d;
     cudaStream_t st = args_.stream;
     const double s_ref = 1.0 / 3.0;
-    const double* total;
-    if (maps_ok_ && !iso_ && ix32_) {
+    const double* total = nullptr;
+    if (!kCell && maps_ok_ && !iso_ && ix32_) {
+      if constexpr (!kCell) {
       // one pass of the fused lb kernel in its observing form over this
       // lattice's tiles (the step's tile machinery, nothing stored)
       // the lattice's tiles in the chunk list the step runs with (the
@@ -833,6 +868,7 @@ class Engine final : public EngineBase {
                                              I.obs_part + (int64_t)I.obs_ntiles * OBS_SLOTS);
       NLC_CK_LAUNCH("k_obs_final");
       total = I.obs_part + (int64_t)I.obs_ntiles * OBS_SLOTS;
+      }
     } else {
       // stress of the current Q, then rho, u and the observables in one pass
       k_stress<Lat, T><<<grid1(n), 256, 0, st>>>(I.q[cur_], I.pi, I.d, I.p, iso_);
@@ -911,11 +947,107 @@ class Engine final : public EngineBase {
     if (I.pi) return NLC_OK;
     nlc_status s;
     const int64_t n = I.d.n;
-    T* qp;
-    if ((s = alloc(&I.pi, (size_t)DIM * DIM * n)) || (s = alloc(&qp, (size_t)5 * I.L.comp)) ||
-        (s = alloc(&I.r1, (size_t)5 * n)))
+    T *pi = nullptr, *qp = nullptr, *r1 = nullptr;
+    if ((s = alloc(&pi, (size_t)DIM * DIM * n)) || (s = alloc(&qp, (size_t)5 * I.L.comp)) ||
+        (s = alloc(&r1, (size_t)5 * n))) {
+      release(pi);
+      release(qp);
       return s;
+    }
+    I.pi = pi;
     I.qp = Field<T>{qp, I.L};
+    I.r1 = r1;
+    return NLC_OK;
+  }
+
+  // gives one allocation back (nothing for nullptr)
+  void release(void* p) {
+    if (!p) return;
+    cudaFree(p);
+    allocs_.erase(std::remove(allocs_.begin(), allocs_.end(), p), allocs_.end());
+  }
+
+  // float64 arithmetic: the workspaces (those of the unfused schedule) and
+  // descriptors of the cell kernels.  Where the workspaces do not fit on the
+  // device (set_fields and read-back need them too, so only for a context
+  // that is filled by load_state), the steps keep the tiled kernels, which
+  // need none.
+  nlc_status ensure_cells() {
+    if constexpr (kCell) {
+      if (cells_off_ || (cells_dev_ && !cells_stale_)) return NLC_OK;
+      nlc_status s;
+      const size_t n = inst_.size();
+      for (size_t i = 0; i < n; i++) {
+        s = ensure_unfused(inst_[i]);
+        if (s == NLC_ENOMEM) {
+          cells_off_ = true;
+          err.clear();
+          return NLC_OK;
+        }
+        if (s) return s;
+      }
+      if (!cells_dev_ && (s = alloc(&cells_dev_, n))) return s;
+      if (any_mrt_ && !cell_mrt_ && (s = alloc(&cell_mrt_, n * Q))) return s;
+      std::vector<CellInst<G>> ci(n);
+      std::vector<double> rates(n * Q, 0.0);
+      int64_t nb = 0;
+      for (size_t i = 0; i < n; i++) {
+        InstHost<T, G>& I = inst_[i];
+        CellInst<G>& C = ci[i];
+        C.d = I.d;
+        C.L = I.L;
+        C.c = make_cell_par<Lat>(I.p, iso_);
+        for (int b = 0; b < 2; b++) {
+          C.g[b] = I.g[b];
+          C.q[b] = I.q[b].base;
+        }
+        C.u = I.u.base;
+        C.pi = I.pi;
+        C.h = I.r1;
+        C.qp = I.qp.base;
+        C.mrt = mrt_on_[i] ? cell_mrt_ + i * Q : nullptr;
+        for (int k = 0; k < Q && mrt_on_[i]; k++)
+          rates[i * Q + k] = I.mrt_coef[k] * mrt_group_factor<Lat>(k);
+        C.block0 = (unsigned)nb;
+        nb += (I.d.n + CELL_T - 1) / CELL_T;
+      }
+      if (nb > INT32_MAX) {
+        cells_off_ = true;
+        return NLC_OK;
+      }
+      cell_blocks_ = (unsigned)nb;
+      cudaStream_t st = args_.stream;
+      if (any_mrt_)
+        NLC_CK(cudaMemcpyAsync(cell_mrt_, rates.data(), sizeof(double) * n * Q,
+                               cudaMemcpyHostToDevice, st));
+      NLC_CK(cudaMemcpyAsync(cells_dev_, ci.data(), sizeof(CellInst<G>) * n,
+                             cudaMemcpyHostToDevice, st));
+      NLC_CK(cudaStreamSynchronize(st));
+      cells_stale_ = false;
+    }
+    return NLC_OK;
+  }
+
+  // one step of every lattice: the four cell kernels
+  nlc_status step_cells(cudaStream_t st) {
+    if constexpr (kCell) {
+      int e[5];
+      auto at = [&](int k) { e[k] = mark(); };
+      const cudaError_t r =
+          iso_ ? launch_cell_step<Lat, G, true>(cells_dev_, (int)inst_.size(), cell_blocks_, cur_,
+                                                st, at)
+               : launch_cell_step<Lat, G, false>(cells_dev_, (int)inst_.size(), cell_blocks_, cur_,
+                                                 st, at);
+      if (r != cudaSuccess) {
+        err = std::string("cell kernels: ") + cudaGetErrorString(r);
+        return NLC_ECUDA;
+      }
+      if (timer.on) {
+        const int kid[4] = {KID_STRESS, KID_LB, KID_PREDICT, KID_CORRECT};
+        for (int k = 0; k < 4; k++) timer.span(kid[k], e[k], e[k + 1]);
+      }
+      cur_ ^= 1;
+    }
     return NLC_OK;
   }
 
@@ -1218,6 +1350,7 @@ class Engine final : public EngineBase {
 
   // one step of every lattice: two launches over the joint tile list
   nlc_status step_fused(cudaStream_t st) {
+    if (cells_dev_ && !cells_off_) return step_cells(st);
     const int a = cur_;
     const int e0 = mark();
     cudaError_t e = launch_fused_lb<Lat, T>(insts_dev_, qmaps_dev_, tiles_dev_, ntiles_, a,
@@ -1246,6 +1379,8 @@ class Engine final : public EngineBase {
   // replay a captured graph of exactly len steps (cached per buffer parity
   // and length) instead of launching kernel by kernel
   nlc_status fused_steps(int64_t len) {
+    nlc_status cs = ensure_cells();
+    if (cs) return cs;
     if (len < 4 || timer.on) {
       for (int64_t j = 0; j < len; j++) {
         nlc_status s = step_fused(args_.stream);
@@ -1276,6 +1411,8 @@ class Engine final : public EngineBase {
       nlc_status ps = persist_grid(&grid);
       if (ps) return ps;
     }
+    nlc_status cs = ensure_cells();
+    if (cs) return cs;
     const int saved = cur_;
     cur_ = c;
     NLC_CK(cudaStreamBeginCapture(cap_stream_, cudaStreamCaptureModeThreadLocal));
@@ -1327,6 +1464,12 @@ class Engine final : public EngineBase {
   bool taper_ = false;  // tapered chunk lists (chunk_bounds)
   int ntiles_ = 0;
   bool maps_ok_ = false;
+  // float64 arithmetic: descriptors of the cell kernels (ensure_cells)
+  CellInst<G>* cells_dev_ = nullptr;
+  double* cell_mrt_ = nullptr;   // [lattices][Q]
+  unsigned cell_blocks_ = 0;
+  bool cells_stale_ = true;      // to be uploaded before the next step
+  bool cells_off_ = false;       // workspaces do not fit: tiled kernels
   unsigned long long* bad_ = nullptr;
   unsigned* derr_ = nullptr;
   int cur_ = 0;

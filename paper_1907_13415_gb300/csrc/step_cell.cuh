@@ -1,0 +1,581 @@
+// step_cell.cuh -- the time step for float64 arithmetic (NLC_FP64 and
+// NLC_FP32_QF64): four one-cell-per-thread kernels.
+//
+// GB300 issues float64 instructions at a small fraction of its float32 rate
+// (measured: one warp instruction every 19 clocks per SM with four or more
+// warps, one every 64 clocks for a single warp, whatever the number of
+// active lanes), so these steps are bound by the number of float64
+// instructions and by how evenly they spread over the SMs; integer work,
+// loads and DRAM traffic are nearly free beside them.  Hence, other than in
+// the tiled float32 kernels (step_fused.cuh):
+//   - nothing is computed twice: no ring recomputation (1.33 times the
+//     stress and the predictor there); intermediates go through memory, and
+//     the molecular field that the stress needs is kept for the predictor;
+//   - the pointwise formulas below are rearranged for few instructions:
+//     factors 1/2 and the stencils' weights go into constants formed once
+//     per lattice (CellPar), the collision works on sums and differences of
+//     opposite populations, Q Q and the gradient products use tracelessness;
+//   - blocks of one warp over the linear cell index, so that small lattices
+//     reach as many SMs as they have warps and large ones leave no tail
+//     (two warps: 2-6% slower between 5,000 and 30,000 cells, else the same).
+// Float64 instructions per cell: D2Q9 114 + 79 + 71 + 120, D3Q19 175 + 156 +
+// 113 + 171.  Measured, tiled kernels -> these (us per step): 128 x 8 D2Q9
+// 55 -> 20, 256^2 D2Q9 114 -> 56 (48 at the issue rate above), 64^3 D3Q19
+// 830 -> 311 (300 at that rate; with float populations, whose conversions
+// run in integer arithmetic below, 312 instead of 329).
+#pragma once
+#include <cstring>
+
+#include "common.cuh"
+#include "lattice.cuh"
+#include "mrt.cuh"
+#include "packed.cuh"
+#include "physics.cuh"
+#include "step_fused.cuh"
+#include "step_unfused.cuh"
+#include "tma.cuh"
+
+namespace nlc {
+
+constexpr int CELL_T = 32;  // threads per block: one warp
+
+// Constants of one lattice.  The stencils give plain differences d~ and sums
+// s~ of neighbours (cell_stencil) with grad = gs/2 d~ and
+// lap = gs s~ - ls v; gs = 1, ls = 2 DIM for the standard stencils.
+struct CellPar {
+  double rho0, inv_tau, keep;     // keep = 1 - 1/tau
+  double A1, Ag, Ag3, Kg;         // Eq. 3: A1 = -A0 (1 - gamma/3) - K ls, Kg = K gs
+  double s2, s23, sm, sp, sK;     // Eq. 5 times gs/2 (the stress is stored so scaled:
+                                  // F = sum of its plain differences)
+  double xi, x2, Gamma, hs, qs, hu;  // Eq. 1: hs = gs/2, qs = gs/4, hu = -gs/2
+  double cC, cR, cB, cG;          // BGK: w2/tau, 3 w2/tau, 9 w2 k, 3 w2 k, k = 1 - 1/(2 tau)
+};
+
+template <class Lat>
+inline CellPar make_cell_par(const Par<double>& p, bool iso) {
+  constexpr double w2 = 1.0 / 36.0, w1 = Lat::DIM == 2 ? 1.0 / 9.0 : 1.0 / 18.0;
+  const double gs = iso ? 6.0 * w1 : 1.0;
+  const double ls = iso ? 6.0 * (1.0 - Lat::w(0)) : 2.0 * Lat::DIM;
+  CellPar c;
+  c.rho0 = p.rho0;
+  c.inv_tau = p.inv_tau;
+  c.keep = 1.0 - p.inv_tau;
+  c.A1 = p.A1 - p.K * ls;
+  c.Ag = p.Ag;
+  c.Ag3 = p.Ag3;
+  c.Kg = p.K * gs;
+  const double f = 0.5 * gs;
+  c.s2 = f * p.x2;
+  c.s23 = f * p.x23;
+  c.sm = f * p.xm1;
+  c.sp = f * p.xp1;
+  c.sK = f * (p.K * gs * gs * 0.5);
+  c.xi = p.xi;
+  c.x2 = p.x2;
+  c.Gamma = p.Gamma;
+  c.hs = 0.5 * gs;
+  c.qs = 0.25 * gs;
+  c.hu = -0.5 * gs;
+  c.cC = w2 * p.inv_tau;
+  c.cR = 3.0 * w2 * p.inv_tau;
+  c.cB = 9.0 * w2 * p.guo;
+  c.cG = 3.0 * w2 * p.guo;
+  return c;
+}
+
+// One lattice as the cell kernels see it.
+template <class G>
+struct CellInst {
+  Dims d;
+  Layout L;
+  CellPar c;
+  G* g[2];
+  double* q[2];   // padded Q, ping-pong
+  double* u;      // padded u^n
+  double* pi;     // stress times gs/2, dense [DIM DIM][n]
+  double* h;      // H(Q^n) for the predictor, then Q^n + Q^P for the corrector, dense [5][n]
+  double* qp;     // padded predictor Q^P
+  const double* mrt;  // coefficients of collide_mrt_groups, or nullptr (BGK)
+  unsigned block0;    // first block of this lattice in the launch
+};
+
+// Plain differences d[a] along each axis and the sum s of the neighbours of
+// the value at p[0]; sy, sz: strides of y and z.  ISO: the lattice's own
+// neighbour set, diagonal neighbours with their weight relative to the axis
+// ones (1/4 on D2Q9, 1/2 on D3Q19).
+template <class Lat, bool ISO>
+__device__ __forceinline__ void cell_stencil(const double* __restrict__ p, int64_t sy, int64_t sz,
+                                             double d[3], double& s) {
+  constexpr int DIM = Lat::DIM;
+  const double xp = p[1], xm = p[-1], yp = p[sy], ym = p[-sy];
+  d[0] = xp - xm;
+  d[1] = yp - ym;
+  d[2] = 0.0;
+  s = (xp + xm) + (yp + ym);
+  if constexpr (DIM == 3) {
+    const double zp = p[sz], zm = p[-sz];
+    d[2] = zp - zm;
+    s += zp + zm;
+  }
+  if constexpr (ISO) {
+    constexpr double r = DIM == 2 ? 0.25 : 0.5;
+    double t = 0.0, e[3] = {0.0, 0.0, 0.0};
+    auto quad = [&](int64_t sa, int64_t sb, int a, int b) {
+      const double pp = p[sa + sb], mm = p[-sa - sb], pm = p[sa - sb], mp = p[sb - sa];
+      const double u = pp - mm, v = pm - mp;
+      e[a] += u + v;
+      e[b] += u - v;
+      t += (pp + mm) + (pm + mp);
+    };
+    quad(1, sy, 0, 1);
+    if constexpr (DIM == 3) {
+      quad(1, sz, 0, 2);
+      quad(sy, sz, 1, 2);
+    }
+#pragma unroll
+    for (int a = 0; a < DIM; a++) d[a] = fma(r, e[a], d[a]);
+    s = fma(r, t, s);
+  }
+}
+
+// H of Eq. 3 from q and the neighbour sums s (the Laplacian's centre term is
+// in c.A1).  Q Q of a traceless Q: (QQ)_xy = c e - b f, (QQ)_xz = b e - c d,
+// (QQ)_yz = b c - a e with f = Qzz.
+__host__ __device__ __forceinline__ void cell_field(const double q[5], const double s[5], const CellPar& c,
+                                           double h[5]) {
+  const double a = q[0], b = q[1], cc = q[2], d = q[3], e = q[4], f = -(a + d);
+  const double b2 = b * b, c2 = cc * cc, e2 = e * e;
+  const double q0 = fma(a, a, b2 + c2), q3 = fma(d, d, b2 + e2), q5 = fma(f, f, c2 + e2);
+  const double q1 = fma(cc, e, -(b * f)), q2 = fma(b, e, -(cc * d)), q4 = fma(b, cc, -(a * e));
+  const double tr2 = (q0 + q3) + q5;
+  const double c1 = fma(-c.Ag, tr2, c.A1), c3 = c.Ag3 * tr2;
+  h[0] = fma(c1, a, fma(c.Ag, q0, fma(c.Kg, s[0], c3)));
+  h[1] = fma(c1, b, fma(c.Ag, q1, c.Kg * s[1]));
+  h[2] = fma(c1, cc, fma(c.Ag, q2, c.Kg * s[2]));
+  h[3] = fma(c1, d, fma(c.Ag, q3, fma(c.Kg, s[3], c3)));
+  h[4] = fma(c1, e, fma(c.Ag, q4, c.Kg * s[4]));
+}
+
+// Eq. 5 without P0 (see physics.cuh: stress), times gs/2, from the plain
+// differences d[g][k].  d_aQ : d_bQ = 2 sum_k A_k B'_k with B'_0 = B_0 + B_3/2,
+// B'_3 = B_3 + B_0/2, B'_k = B_k otherwise.
+template <int DIM>
+__host__ __device__ __forceinline__ void cell_stress(const double q[5], const double h[5],
+                                            const double d[3][5], const CellPar& c,
+                                            double P[3][3]) {
+  const double Q[3][3] = {{q[0], q[1], q[2]}, {q[1], q[3], q[4]}, {q[2], q[4], -(q[0] + q[3])}};
+  const double H[3][3] = {{h[0], h[1], h[2]}, {h[1], h[3], h[4]}, {h[2], h[4], -(h[0] + h[3])}};
+  double X[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; a++)
+#pragma unroll
+    for (int b = 0; b < 3; b++)
+      if ((a < DIM && b < DIM) || (a == 2 && b == 2))
+        X[a][b] = fma(Q[a][0], H[0][b], fma(Q[a][1], H[1][b], Q[a][2] * H[2][b]));
+  const double xq = c.s2 * ((X[0][0] + X[1][1]) + X[2][2]);
+  const double xq3 = xq * (1.0 / 3.0);
+#pragma unroll
+  for (int b = 0; b < DIM; b++) {
+    const double B0 = fma(0.5, d[b][3], d[b][0]), B3 = fma(0.5, d[b][0], d[b][3]);
+#pragma unroll
+    for (int a = 0; a <= b; a++) {
+      const double el =
+          fma(d[a][0], B0,
+              fma(d[a][3], B3,
+                  fma(d[a][1], d[b][1], fma(d[a][2], d[b][2], d[a][4] * d[b][4]))));
+      if (a == b) {
+        const double t = fma(xq, Q[a][a], fma(-c.s23, H[a][a], fma(-c.sK, el, xq3)));
+        P[a][a] = fma(-c.s2, X[a][a], t);
+      } else {
+        const double t = fma(xq, Q[a][b], fma(-c.s23, H[a][b], -(c.sK * el)));
+        P[a][b] = fma(-c.sm, X[a][b], fma(-c.sp, X[b][a], t));
+        P[b][a] = fma(-c.sm, X[b][a], fma(-c.sp, X[a][b], t));
+      }
+    }
+  }
+}
+
+// r = base + R of Eq. 1 with its trace projected out (see physics.cuh:
+// be_rhs_adv), from q, h = H, the plain differences d of Q and g[a][b] of u_a
+// along b, and u.  With N = 4/gs (xi D + W): N_aa = 2 xi g_aa,
+// N_ab = xi p + m, N_ba = xi p - m, p, m = g_ab +- g_ba.
+template <int DIM>
+__host__ __device__ __forceinline__ void cell_rhs(const double q[5], const double h[5],
+                                         const double d[3][5], const double u[3],
+                                         const double g[3][3], const CellPar& c,
+                                         const double base[5], double r[5]) {
+  constexpr bool D3 = DIM == 3;
+  const double third = 1.0 / 3.0;
+  const double t00 = q[0] + third, t11 = q[3] + third, t22 = third - (q[0] + q[3]);
+  const double b = q[1], cc = q[2], e = q[4];
+  const double n00 = c.x2 * g[0][0], n11 = c.x2 * g[1][1], n22 = D3 ? c.x2 * g[2][2] : 0.0;
+  const double p01 = g[0][1] + g[1][0], m01 = g[0][1] - g[1][0];
+  const double N01 = fma(c.xi, p01, m01), N10 = fma(c.xi, p01, -m01);
+  double N02 = 0.0, N20 = 0.0, N12 = 0.0, N21 = 0.0, off = b * p01;
+  if constexpr (D3) {
+    const double p02 = g[0][2] + g[2][0], m02 = g[0][2] - g[2][0];
+    const double p12 = g[1][2] + g[2][1], m12 = g[1][2] - g[2][1];
+    N02 = fma(c.xi, p02, m02), N20 = fma(c.xi, p02, -m02);
+    N12 = fma(c.xi, p12, m12), N21 = fma(c.xi, p12, -m12);
+    off = fma(cc, p02, fma(e, p12, off));
+  }
+  // 2 xi Q:G^T over gs/2, and the trace 2 xi div u / 3 over gs/2
+  const double tau = fma(q[0], D3 ? n00 - n22 : n00, fma(q[3], D3 ? n11 - n22 : n11, c.x2 * off));
+  const double tr = (D3 ? (n00 + n11) + n22 : n00 + n11) * (-1.0 / 9.0);
+  const double a0 = n00 - tau, a1 = n11 - tau, a2 = D3 ? n22 - tau : -tau;
+  double S[5];
+  S[0] = fma(a0, t00, fma(N01, b, tr));
+  S[3] = fma(a1, t11, fma(N10, b, tr));
+  S[1] = fma(a0 + a1, b, fma(N01, t11, N10 * t00));
+  if constexpr (D3) {
+    S[0] = fma(N02, cc, S[0]);
+    S[3] = fma(N12, e, S[3]);
+    S[1] = fma(N02, e, fma(N12, cc, S[1]));
+    S[2] = fma(a0 + a2, cc, fma(N01, e, fma(N02, t22, fma(N20, t00, N21 * b))));
+    S[4] = fma(a1 + a2, e, fma(N10, cc, fma(N12, t22, fma(N20, b, N21 * t11))));
+  } else {
+    S[2] = fma(a0 + a2, cc, N01 * e);
+    S[4] = fma(a1 + a2, e, N10 * cc);
+  }
+  const double u0 = c.hu * u[0], u1 = c.hu * u[1], u2 = D3 ? c.hu * u[2] : 0.0;
+#pragma unroll
+  for (int k = 0; k < 5; k++) {
+    double v = fma(c.Gamma, h[k], base[k]);
+    if constexpr (D3) v = fma(u2, d[2][k], v);
+    v = fma(u1, d[1][k], fma(u0, d[0][k], v));
+    r[k] = fma(k == 0 || k == 3 ? c.hs : c.qs, S[k], v);
+  }
+}
+
+__host__ __device__ __forceinline__ unsigned float_bits(float v) {
+#ifdef __CUDA_ARCH__
+  return __float_as_uint(v);
+#else
+  unsigned b;
+  memcpy(&b, &v, 4);
+  return b;
+#endif
+}
+__host__ __device__ __forceinline__ float float_of(unsigned b) {
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(b);
+#else
+  float v;
+  memcpy(&v, &b, 4);
+  return v;
+#endif
+}
+__host__ __device__ __forceinline__ double double_of(unsigned hi, unsigned lo) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double((int)hi, (int)lo);
+#else
+  const uint64_t b = ((uint64_t)hi << 32) | lo;
+  double v;
+  memcpy(&v, &b, 8);
+  return v;
+#endif
+}
+__host__ __device__ __forceinline__ unsigned hi_word(double v) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)__double2hiint(v);
+#else
+  uint64_t b;
+  memcpy(&b, &v, 8);
+  return (unsigned)(b >> 32);
+#endif
+}
+__host__ __device__ __forceinline__ unsigned lo_word(double v) {
+#ifdef __CUDA_ARCH__
+  return (unsigned)__double2loint(v);
+#else
+  uint64_t b;
+  memcpy(&b, &v, 8);
+  return (unsigned)b;
+#endif
+}
+
+// Exact float -> double in integer arithmetic (conversions to and from
+// 64-bit types run at the float64 rate).  Denormals count as zero, as in the
+// rest of the float32 code (-ftz).
+__host__ __device__ __forceinline__ double widen(float v) {
+  const unsigned b = float_bits(v), m = b & 0x7fffffffu;
+  unsigned hi = (m >> 3) + 0x38000000u;           // rebias 127 -> 1023
+  hi = m >= 0x7f800000u ? hi + 0x38000000u : hi;  // infinities and NaN
+  hi = m < 0x00800000u ? 0u : hi;
+  const unsigned lo = m < 0x00800000u ? 0u : b << 29;
+  return double_of(hi | (b & 0x80000000u), lo);
+}
+__host__ __device__ __forceinline__ double widen(double v) { return v; }
+
+// The nearest float (ties to even), likewise in integer arithmetic; results
+// below the normal range are zero.
+__host__ __device__ __forceinline__ float narrow(double v) {
+  const unsigned hi = hi_word(v), lo = lo_word(v), m = hi & 0x7fffffffu;
+  unsigned f = ((m - 0x38000000u) << 3) | (lo >> 29);
+  const unsigned rest = lo & 0x1fffffffu;
+  f += (rest > 0x10000000u || (rest == 0x10000000u && (f & 1u))) ? 1u : 0u;
+  f = m < 0x38100000u ? 0u : f;                                // below 2^-126
+  f = m >= 0x47f00000u ? 0x7f800000u : f;                      // 2^128 and above
+  f = m > 0x7ff00000u || (m == 0x7ff00000u && lo) ? 0x7fffffffu : f;  // NaN
+  return float_of(f | (hi & 0x80000000u));
+}
+template <class G>
+__host__ __device__ __forceinline__ G store_as(double v) {
+  if constexpr (sizeof(G) == 4)
+    return narrow(v);
+  else
+    return v;
+}
+
+// The lattice and cell of this thread: block b of the launch holds cells
+// CELL_T (b - block0) .. of the lattice whose block range it falls in.
+template <class G>
+__device__ __forceinline__ bool cell_decode(const CellInst<G>* __restrict__ insts, int ninst,
+                                            const CellInst<G>*& I, int64_t& idx, int& x, int& y,
+                                            int& z) {
+  int lo = 0, hi = ninst;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    (insts[mid].block0 <= blockIdx.x ? lo : hi) = mid;
+  }
+  I = insts + lo;
+  idx = (int64_t)(blockIdx.x - I->block0) * CELL_T + threadIdx.x;
+  return decode(I->d, idx, x, y, z);
+}
+
+// 1. H and the stress of Q^n
+template <class Lat, class G, bool ISO>
+__global__ void __launch_bounds__(CELL_T) k_cell_stress(const CellInst<G>* __restrict__ insts,
+    int ninst, int cur) {
+  constexpr int DIM = Lat::DIM;
+  grid_dep_wait();
+  const CellInst<G>* I;
+  int64_t idx;
+  int x, y, z;
+  if (!cell_decode(insts, ninst, I, idx, x, y, z)) return;
+  const CellPar c = I->c;
+  const Field<double> Q{I->q[cur], I->L};
+  const double* p = Q.base + Q.off(0, x, y, z);
+  double q[5], d[3][5], s[5], h[5], P[3][3];
+#pragma unroll
+  for (int k = 0; k < 5; k++) {
+    double dk[3];
+    q[k] = p[k * Q.L.comp];
+    cell_stencil<Lat, ISO>(p + k * Q.L.comp, Q.L.nxp, Q.L.plane, dk, s[k]);
+    d[0][k] = dk[0], d[1][k] = dk[1], d[2][k] = dk[2];
+  }
+  cell_field(q, s, c, h);
+  cell_stress<DIM>(q, h, d, c, P);
+  const int64_t n = I->d.n;
+#pragma unroll
+  for (int k = 0; k < 5; k++) I->h[k * n + idx] = h[k];
+#pragma unroll
+  for (int a = 0; a < DIM; a++)
+#pragma unroll
+    for (int b = 0; b < DIM; b++) I->pi[(a * DIM + b) * n + idx] = P[a][b];
+}
+
+// 2. F, the pulled populations, rho and u, the collision
+template <class Lat, class G, bool ISO>
+__global__ void __launch_bounds__(CELL_T) k_cell_lb(const CellInst<G>* __restrict__ insts,
+    int ninst, int cur) {
+  constexpr int DIM = Lat::DIM, NP = (Lat::Q - 1) / 2;
+  grid_dep_wait();
+  const CellInst<G>* I;
+  int64_t idx;
+  int x, y, z;
+  if (!cell_decode(insts, ninst, I, idx, x, y, z)) return;
+  const CellPar c = I->c;
+  const Dims d = I->d;
+  // periodic neighbours: source offsets along each axis, index c + 1
+  const int64_t nx = d.nx, nxy = nx * d.ny;
+  const int64_t col[3] = {wrap_dec(x, d.nx), x, wrap_inc(x, d.nx)};
+  const int64_t row[3] = {wrap_dec(y, d.ny) * nx, y * nx, wrap_inc(y, d.ny) * nx};
+  const int64_t pl[3] = {DIM == 3 ? wrap_dec(z, d.nz) * nxy : z * nxy, z * nxy,
+                         DIM == 3 ? wrap_inc(z, d.nz) * nxy : z * nxy};
+  auto at = [&](int cx, int cy, int cz) { return pl[cz + 1] + row[cy + 1] + col[cx + 1]; };
+  const G* __restrict__ gin = I->g[cur];
+  G* __restrict__ gout = I->g[cur ^ 1];
+  double g0 = widen(gin[idx]), gi[NP], gj[NP];
+#pragma unroll
+  for (int k = 0; k < NP; k++) {
+    const int i = pair_first<Lat>(k), j = Lat::opp(i);
+    gi[k] = widen(gin[i * d.n + at(-Lat::c(i, 0), -Lat::c(i, 1), -Lat::c(i, 2))]);
+    gj[k] = widen(gin[j * d.n + at(Lat::c(i, 0), Lat::c(i, 1), Lat::c(i, 2))]);
+  }
+  double F[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int a = 0; a < DIM; a++) {
+    double s = 0.0, t = 0.0;
+#pragma unroll
+    for (int b = 0; b < DIM; b++) {
+      const double* __restrict__ P = I->pi + (a * DIM + b) * d.n;
+      const int ex = b == 0, ey = b == 1, ez = b == 2;
+      const double v = P[at(ex, ey, ez)] - P[at(-ex, -ey, -ez)];
+      s = b == 0 ? v : s + v;
+      if constexpr (ISO) {
+#pragma unroll
+        for (int o = 0; o < DIM; o++) {
+          if (o == b) continue;
+          const int ox = o == 0, oy = o == 1, oz = o == 2;
+          t += (P[at(ex + ox, ey + oy, ez + oz)] - P[at(-ex - ox, -ey - oy, -ez - oz)]) +
+               (P[at(ex - ox, ey - oy, ez - oz)] - P[at(ox - ex, oy - ey, oz - ez)]);
+        }
+      }
+    }
+    F[a] = ISO ? fma(DIM == 2 ? 0.25 : 0.5, t, s) : s;
+  }
+  // sums and differences of opposite populations; rho and u of Eq. 6
+  double rho, drho, J[3], u[3];
+  moments_groups<Lat, double>(g0, gi, gj, F, c.rho0, rho, drho, J, u);
+  auto put = [&](int i, double v) { gout[i * d.n + idx] = store_as<G>(v); };
+  if (I->mrt) {
+    collide_mrt_groups<Lat, double>(g0, gi, gj, rho, drho, J, u, F, I->mrt);
+    put(0, g0);
+#pragma unroll
+    for (int k = 0; k < NP; k++) {
+      put(pair_first<Lat>(k), gi[k]);
+      put(Lat::opp(pair_first<Lat>(k)), gj[k]);
+    }
+  } else {
+    // BGK with the source term (physics.cuh: collide_bgk) over the diagonal
+    // weight w2: even part C + M_aa (+ M_bb +- M_ab), odd part L_a (+- L_b)
+    // with t = A u + B F, M_aa = u_a t_a, M_ab = u_a t_b + u_b t_a and
+    // L = R u + G F; the even part of the axis pairs (the rest population)
+    // carries the weight ratio ra (r0)
+    constexpr double ra = DIM == 2 ? 4.0 : 2.0, r0 = DIM == 2 ? 16.0 : 12.0;
+    const double R = c.cR * rho, A = 1.5 * R;
+    double t[3], L[3], M[3];
+#pragma unroll
+    for (int a = 0; a < DIM; a++) {
+      t[a] = fma(A, u[a], c.cB * F[a]);
+      L[a] = fma(R, u[a], c.cG * F[a]);
+      M[a] = u[a] * t[a];
+    }
+    const double Ms = DIM == 3 ? (M[0] + M[1]) + M[2] : M[0] + M[1];
+    const double C = fma(c.cC, drho, Ms * (-1.0 / 3.0));
+    put(0, fma(c.keep, g0, r0 * C));
+    double B[3];  // C + M_aa
+#pragma unroll
+    for (int a = 0; a < DIM; a++) B[a] = C + M[a];
+#pragma unroll
+    for (int k = 0; k < NP; k++) {
+      const int i = pair_first<Lat>(k), j = Lat::opp(i);
+      int a = -1, b = -1;  // the axes the pair moves along
+#pragma unroll
+      for (int o = 0; o < DIM; o++)
+        if (Lat::c(i, o) != 0) (a < 0 ? a : b) = o;
+      if (b < 0) {
+        put(i, fma(ra, B[a] + L[a], c.keep * gi[k]));
+        put(j, fma(ra, B[a] - L[a], c.keep * gj[k]));
+      } else {
+        const bool same = Lat::c(i, a) == Lat::c(i, b);
+        const double Mab = fma(u[a], t[b], u[b] * t[a]);
+        const double N = B[a] + M[b];
+        const double E = same ? N + Mab : N - Mab;
+        // odd part along c_i
+        double O = same ? L[a] + L[b] : L[a] - L[b];
+        if (Lat::c(i, a) < 0) O = -O;
+        put(i, fma(c.keep, gi[k], E + O));
+        put(j, fma(c.keep, gj[k], E - O));
+      }
+    }
+  }
+  const Field<double> U{I->u, I->L};
+  store_with_images<double, DIM, DIM>(U, d, x, y, z, u);
+}
+
+// q, its plain differences and neighbour sums, u and its plain differences
+template <class Lat, bool ISO>
+__device__ __forceinline__ void cell_load(const double* __restrict__ p,
+                                          const double* __restrict__ pu, const Layout& L,
+                                          double q[5], double d[3][5], double s[5], double u[3],
+                                          double g[3][3]) {
+  constexpr int DIM = Lat::DIM;
+#pragma unroll
+  for (int k = 0; k < 5; k++) {
+    double dk[3];
+    q[k] = p[k * L.comp];
+    cell_stencil<Lat, ISO>(p + k * L.comp, L.nxp, L.plane, dk, s[k]);
+    d[0][k] = dk[0], d[1][k] = dk[1], d[2][k] = dk[2];
+  }
+#pragma unroll
+  for (int a = 0; a < DIM; a++) {
+    double unused;
+    u[a] = pu[a * L.comp];
+    cell_stencil<Lat, ISO>(pu + a * L.comp, L.nxp, L.plane, g[a], unused);
+  }
+}
+
+// 3. predictor Q^P = Q^n + R(Q^n), and Q^n + Q^P for the corrector
+template <class Lat, class G, bool ISO>
+__global__ void __launch_bounds__(CELL_T) k_cell_predict(const CellInst<G>* __restrict__ insts,
+    int ninst, int cur) {
+  constexpr int DIM = Lat::DIM;
+  grid_dep_wait();
+  const CellInst<G>* I;
+  int64_t idx;
+  int x, y, z;
+  if (!cell_decode(insts, ninst, I, idx, x, y, z)) return;
+  const CellPar c = I->c;
+  const Field<double> Q{I->q[cur], I->L};
+  const int64_t o = Q.off(0, x, y, z), n = I->d.n;
+  double q[5], d[3][5], s[5], u[3], g[3][3], h[5], qp[5];
+  cell_load<Lat, ISO>(Q.base + o, I->u + o, Q.L, q, d, s, u, g);
+#pragma unroll
+  for (int k = 0; k < 5; k++) h[k] = I->h[k * n + idx];
+  cell_rhs<DIM>(q, h, d, u, g, c, q, qp);
+#pragma unroll
+  for (int k = 0; k < 5; k++) I->h[k * n + idx] = q[k] + qp[k];
+  store_with_images<double, 5, DIM>(Field<double>{I->qp, I->L}, I->d, x, y, z, qp);
+}
+
+// 4. corrector Q^{n+1} = [Q^n + Q^P + R(Q^P)]/2
+template <class Lat, class G, bool ISO>
+__global__ void __launch_bounds__(CELL_T) k_cell_correct(const CellInst<G>* __restrict__ insts,
+    int ninst, int cur) {
+  constexpr int DIM = Lat::DIM;
+  grid_dep_wait();
+  const CellInst<G>* I;
+  int64_t idx;
+  int x, y, z;
+  if (!cell_decode(insts, ninst, I, idx, x, y, z)) return;
+  const CellPar c = I->c;
+  const Field<double> QP{I->qp, I->L};
+  const int64_t o = QP.off(0, x, y, z), n = I->d.n;
+  double q[5], d[3][5], s[5], u[3], g[3][3], h[5], base[5], r[5];
+  cell_load<Lat, ISO>(QP.base + o, I->u + o, QP.L, q, d, s, u, g);
+#pragma unroll
+  for (int k = 0; k < 5; k++) base[k] = I->h[k * n + idx];
+  cell_field(q, s, c, h);
+  cell_rhs<DIM>(q, h, d, u, g, c, base, r);
+#pragma unroll
+  for (int k = 0; k < 5; k++) r[k] *= 0.5;
+  store_with_images<double, 5, DIM>(Field<double>{I->q[cur ^ 1], I->L}, I->d, x, y, z, r);
+}
+
+// The four kernels of one step of all lattices (insts in device memory),
+// launched with programmatic serialisation but without the early trigger of
+// the tiled kernels: blocks of the next kernel that are placed while this
+// one runs go wherever an SM has room, and the uneven spread costs more than
+// the launch gap (256^2 D2Q9: 90 us per step with the trigger, 56 without,
+// 57 with plain launches).
+// mark(k) is called before kernel k and mark(4) after the last.
+template <class Lat, class G, bool ISO, class Mark>
+cudaError_t launch_cell_step(const CellInst<G>* insts, int ninst, unsigned nblocks, int cur,
+                             cudaStream_t st, Mark mark) {
+  int k = 0;
+  auto run = [&](auto kernel) {
+    mark(k++);
+    return launch_pdl(kernel, (int)nblocks, CELL_T, 0, st, insts, ninst, cur);
+  };
+  cudaError_t e;
+  if ((e = run(k_cell_stress<Lat, G, ISO>)) != cudaSuccess) return e;
+  if ((e = run(k_cell_lb<Lat, G, ISO>)) != cudaSuccess) return e;
+  if ((e = run(k_cell_predict<Lat, G, ISO>)) != cudaSuccess) return e;
+  if ((e = run(k_cell_correct<Lat, G, ISO>)) != cudaSuccess) return e;
+  mark(4);
+  return cudaSuccess;
+}
+
+}  // namespace nlc

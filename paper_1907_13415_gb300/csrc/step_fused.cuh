@@ -38,6 +38,7 @@
 #include "common.cuh"
 #include "grid_sync.cuh"
 #include "lattice.cuh"
+#include "mrt.cuh"
 #include "packed.cuh"
 #include "physics.cuh"
 #include "step_unfused.cuh"
@@ -343,10 +344,9 @@ __device__ __forceinline__ bool fused_lb_tile(const TileRef tile,
 
   __shared__ T s_mrt[MRT ? Lat::Q : 1];
   if constexpr (MRT) {
-    if (tid < Lat::Q) {
-      constexpr MomentBasis<Lat> B = make_moment_basis<Lat>();
-      s_mrt[tid] = I.mrt ? I.mrt[tid] : T(double(p.inv_tau) / B.n2[tid]);
-    }
+    if (tid < Lat::Q)
+      s_mrt[tid] = (I.mrt ? I.mrt[tid] : p.inv_tau / T(mrt_row_norm<Lat>(tid))) *
+                   T(mrt_group_factor<Lat>(tid));
   }
   if (tid == 0) {
     for (int s = 0; s < C::NSQ; s++) mbar_init(&bars[s], 1);
@@ -530,22 +530,26 @@ __device__ __forceinline__ bool fused_lb_tile(const TileRef tile,
     const unsigned n32 = (unsigned)d.n;
     T rho, u[3];
     if constexpr (MRT) {
-      T g[Lat::Q];
+      T g0, gi[NP], gj[NP], drho, J[3];
       if constexpr (kPacked) {
-        g[0] = gn.g0;
+        g0 = gn.g0;
 #pragma unroll
-        for (int q = 0; q < NP; q++) {
-          g[pair_first<Lat>(q)] = gn.gp[q].x;
-          g[Lat::opp(pair_first<Lat>(q))] = gn.gp[q].y;
-        }
+        for (int q = 0; q < NP; q++) gi[q] = gn.gp[q].x, gj[q] = gn.gp[q].y;
       } else {
+        g0 = gn.g[0];
 #pragma unroll
-        for (int i = 0; i < Lat::Q; i++) g[i] = gn.g[i];
+        for (int q = 0; q < NP; q++)
+          gi[q] = gn.g[pair_first<Lat>(q)], gj[q] = gn.g[Lat::opp(pair_first<Lat>(q))];
       }
-      moments<Lat, T>(g, F, p, rho, u);
-      collide_mrt<Lat, T>(g, rho, u, F, p, s_mrt);
+      moments_groups<Lat, T>(g0, gi, gj, F, p.rho0, rho, drho, J, u);
+      collide_mrt_groups<Lat, T>(g0, gi, gj, rho, drho, J, u, F, s_mrt);
+      gout[o] = G(g0);
 #pragma unroll
-      for (int i = 0; i < Lat::Q; i++) gout[pop_off<IX32>(i, n32, o)] = G(g[i]);
+      for (int q = 0; q < NP; q++) {
+        const int i = pair_first<Lat>(q);
+        gout[pop_off<IX32>(i, n32, o)] = G(gi[q]);
+        gout[pop_off<IX32>(Lat::opp(i), n32, o)] = G(gj[q]);
+      }
     } else if constexpr (kPacked) {
       float g0 = gn.g0, drho;
       float2 gp[NP];
@@ -1280,8 +1284,8 @@ cudaError_t launch_fused_obs(const InstDev<T, G>* insts, const CUtensorMap* qmap
 }
 
 // mrt: MRT collision; iso: isotropic stencils; ix32: every lattice of the
-// launch has Q n < 2^32 (32-bit population offsets, taken by the BGK
-// kernel with the standard stencils)
+// launch has Q n < 2^32 (32-bit population offsets, taken by the kernels
+// with the standard stencils)
 template <class Lat, class T, class G>
 cudaError_t launch_fused_lb(const InstDev<T, G>* insts, const CUtensorMap* qmaps,
                             const TileRef* tiles, int ntiles, int cur, unsigned* err,
@@ -1292,8 +1296,10 @@ cudaError_t launch_fused_lb(const InstDev<T, G>* insts, const CUtensorMap* qmaps
                : launch_fused_lb_as<Lat, T, G, false, true, false>(insts, qmaps, tiles, ntiles,
                                                                    cur, err, st);
   if (mrt)
-    return launch_fused_lb_as<Lat, T, G, true, false, false>(insts, qmaps, tiles, ntiles, cur,
-                                                             err, st);
+    return ix32 ? launch_fused_lb_as<Lat, T, G, true, false, true>(insts, qmaps, tiles, ntiles,
+                                                                   cur, err, st)
+                : launch_fused_lb_as<Lat, T, G, true, false, false>(insts, qmaps, tiles, ntiles,
+                                                                    cur, err, st);
   return ix32 ? launch_fused_lb_as<Lat, T, G, false, false, true>(insts, qmaps, tiles, ntiles,
                                                                   cur, err, st)
               : launch_fused_lb_as<Lat, T, G, false, false, false>(insts, qmaps, tiles, ntiles,

@@ -117,6 +117,21 @@ __host__ __device__ __forceinline__ float grad_dot(const float A[5], const float
 }
 #endif
 
+// A_0 B0 + A_3 B3 + A_1 B_1 + A_2 B_2 + A_4 B_4
+template <class T>
+__host__ __device__ __forceinline__ T dot5(const T A[5], T B0, T B3, const T B[5]) {
+  return fma_(A[0], B0, fma_(A[3], B3, fma_(A[1], B[1], fma_(A[2], B[2], A[4] * B[4]))));
+}
+#ifdef __CUDACC__
+// FP32: four of the products on packed pairs (packed.cuh)
+__host__ __device__ __forceinline__ float dot5(const float A[5], float B0, float B3,
+                                               const float B[5]) {
+  float2 s2 = pmul(pk(A[0], A[3]), pk(B0, B3));
+  s2 = pfma(pk(A[1], A[2]), pk(B[1], B[2]), s2);
+  return fma_(A[4], B[4], s2.x + s2.y);
+}
+#endif
+
 // Eq. 5 without P0, with dF/d(d_b Q) = K d_b Q:
 //   Pi_ab = 2 xi Qt_ab (Q:H) - xi (H Qt)_ab - xi (Qt H)_ab
 //           - K d_a Q : d_b Q + (Q H)_ab - (H Q)_ab,      Qt = Q + I/3.
@@ -196,6 +211,124 @@ template <class T>
 __host__ __device__ __forceinline__ void corotation(const T G[3][3], const T q[5], T xi,
                                                     T s[5]) {
   corotation(G, q, (xi + T(1)) * T(0.5), (xi - T(1)) * T(0.5), T(2) * xi, s);
+}
+
+// ---------------------------------------------------------------------------
+// The same quantities in the fewest operations, for the step kernels, which
+// are bound by instruction issue (float32) or by the float64 rate.  They take
+// plain differences of neighbours d[a][k] (grad = gs/2 d; gs = 1 for the
+// standard stencils), and use that Q and H are traceless.
+// ---------------------------------------------------------------------------
+
+// H of Eq. 3 as A1 q + Kg s + ..., where s carries the Laplacian (s = lap,
+// Kg = K, or neighbour sums with the centre term in A1).  With f = Qzz:
+// (QQ)_xy = c e - b f, (QQ)_xz = b e - c d, (QQ)_yz = b c - a e.
+template <class T>
+__host__ __device__ __forceinline__ void molecular_field_tl(const T q[5], const T s[5], T A1, T Ag,
+                                                            T Ag3, T Kg, T h[5]) {
+  const T a = q[0], b = q[1], c = q[2], d = q[3], e = q[4], f = -(a + d);
+  const T b2 = b * b, c2 = c * c, e2 = e * e;
+  const T q0 = fma_(a, a, b2 + c2), q3 = fma_(d, d, b2 + e2), q5 = fma_(f, f, c2 + e2);
+  const T q1 = fma_(c, e, -(b * f)), q2 = fma_(b, e, -(c * d)), q4 = fma_(b, c, -(a * e));
+  const T tr2 = (q0 + q3) + q5;
+  const T c1 = fma_(-Ag, tr2, A1), c3 = Ag3 * tr2;
+  h[0] = fma_(c1, a, fma_(Ag, q0, fma_(Kg, s[0], c3)));
+  h[1] = fma_(c1, b, fma_(Ag, q1, Kg * s[1]));
+  h[2] = fma_(c1, c, fma_(Ag, q2, Kg * s[2]));
+  h[3] = fma_(c1, d, fma_(Ag, q3, fma_(Kg, s[3], c3)));
+  h[4] = fma_(c1, e, fma_(Ag, q4, Kg * s[4]));
+}
+
+// The stress of Eq. 5 (see stress) with factors x2 = 2 xi, x23 = 2 xi/3,
+// xm1 = xi - 1, xp1 = xi + 1 and K2 = K gs^2/2 (all five may carry a common
+// factor): d_aQ : d_bQ = 2 sum_k A_k B'_k with B'_0 = B_0 + B_3/2,
+// B'_3 = B_3 + B_0/2 and B'_k = B_k otherwise.
+template <class T, int DIM>
+__host__ __device__ __forceinline__ void stress_tl(const T q[5], const T h[5], const T d[3][5],
+                                                   T x2, T x23, T xm1, T xp1, T K2, T P[3][3]) {
+  const T Q[3][3] = {{q[0], q[1], q[2]}, {q[1], q[3], q[4]}, {q[2], q[4], -(q[0] + q[3])}};
+  const T H[3][3] = {{h[0], h[1], h[2]}, {h[1], h[3], h[4]}, {h[2], h[4], -(h[0] + h[3])}};
+  T X[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; a++)
+#pragma unroll
+    for (int b = 0; b < 3; b++)
+      if ((a < DIM && b < DIM) || (a == 2 && b == 2))
+        X[a][b] = fma_(Q[a][0], H[0][b], fma_(Q[a][1], H[1][b], Q[a][2] * H[2][b]));
+  const T xq = x2 * ((X[0][0] + X[1][1]) + X[2][2]);
+  const T xq3 = xq * T(1.0 / 3.0);
+#pragma unroll
+  for (int b = 0; b < DIM; b++) {
+    const T B0 = fma_(T(0.5), d[b][3], d[b][0]), B3 = fma_(T(0.5), d[b][0], d[b][3]);
+#pragma unroll
+    for (int a = 0; a <= b; a++) {
+      const T el = dot5(d[a], B0, B3, d[b]);
+      if (a == b) {
+        const T t = fma_(xq, Q[a][a], fma_(-x23, H[a][a], fma_(-K2, el, xq3)));
+        P[a][a] = fma_(-x2, X[a][a], t);
+      } else {
+        const T t = fma_(xq, Q[a][b], fma_(-x23, H[a][b], -(K2 * el)));
+        P[a][b] = fma_(-xm1, X[a][b], fma_(-xp1, X[b][a], t));
+        P[b][a] = fma_(-xm1, X[b][a], fma_(-xp1, X[a][b], t));
+      }
+    }
+  }
+}
+
+// Co-rotational term of Eq. 1 with the trace of the right-hand side projected
+// out, from the plain differences g[a][b] of u_a along b: components 0 and 3
+// over gs/2, components 1, 2 and 4 over gs/4.  With N = 4/gs (xi D + W):
+// N_aa = 2 xi g_aa, N_ab = xi p + m, N_ba = xi p - m, p, m = g_ab +- g_ba; in
+// two dimensions every term with a z difference drops out (written out,
+// because the compiler may not drop products with zero).
+template <class T, int DIM>
+__host__ __device__ __forceinline__ void corotation_tl(const T q[5], const T g[3][3], T xi, T x2,
+                                                       T S[5]) {
+  constexpr bool D3 = DIM == 3;
+  const T third = T(1.0 / 3.0);
+  const T t00 = q[0] + third, t11 = q[3] + third, t22 = third - (q[0] + q[3]);
+  const T b = q[1], c = q[2], e = q[4];
+  const T n00 = x2 * g[0][0], n11 = x2 * g[1][1], n22 = D3 ? x2 * g[2][2] : T(0);
+  const T p01 = g[0][1] + g[1][0], m01 = g[0][1] - g[1][0];
+  const T N01 = fma_(xi, p01, m01), N10 = fma_(xi, p01, -m01);
+  T N02 = T(0), N20 = T(0), N12 = T(0), N21 = T(0), off = b * p01;
+  if constexpr (D3) {
+    const T p02 = g[0][2] + g[2][0], m02 = g[0][2] - g[2][0];
+    const T p12 = g[1][2] + g[2][1], m12 = g[1][2] - g[2][1];
+    N02 = fma_(xi, p02, m02), N20 = fma_(xi, p02, -m02);
+    N12 = fma_(xi, p12, m12), N21 = fma_(xi, p12, -m12);
+    off = fma_(c, p02, fma_(e, p12, off));
+  }
+  // 2 xi Q:G^T and -2 xi div u / 9 over gs/2
+  const T tau = fma_(q[0], D3 ? n00 - n22 : n00, fma_(q[3], D3 ? n11 - n22 : n11, x2 * off));
+  const T tr = (D3 ? (n00 + n11) + n22 : n00 + n11) * T(-1.0 / 9.0);
+  const T a0 = n00 - tau, a1 = n11 - tau, a2 = D3 ? n22 - tau : -tau;
+  S[0] = fma_(a0, t00, fma_(N01, b, tr));
+  S[3] = fma_(a1, t11, fma_(N10, b, tr));
+  S[1] = fma_(a0 + a1, b, fma_(N01, t11, N10 * t00));
+  if constexpr (D3) {
+    S[0] = fma_(N02, c, S[0]);
+    S[3] = fma_(N12, e, S[3]);
+    S[1] = fma_(N02, e, fma_(N12, c, S[1]));
+    S[2] = fma_(a0 + a2, c, fma_(N01, e, fma_(N02, t22, fma_(N20, t00, N21 * b))));
+    S[4] = fma_(a1 + a2, e, fma_(N10, c, fma_(N12, t22, fma_(N20, b, N21 * t11))));
+  } else {
+    S[2] = fma_(a0 + a2, c, N01 * e);
+    S[4] = fma_(a1 + a2, e, N10 * c);
+  }
+}
+
+// Right-hand side of Eq. 1 (see be_rhs_adv) from twice the advection
+// adv = u . d and the plain differences g of u, gs = 1.
+template <class T, int DIM>
+__host__ __device__ __forceinline__ void be_rhs_tl(const T q[5], const T adv[5], const T lap[5],
+                                                   const T g[3][3], const Par<T>& p, T r[5]) {
+  T h[5], S[5];
+  molecular_field_tl(q, lap, p.A1, p.Ag, p.Ag3, p.K, h);
+  corotation_tl<T, DIM>(q, g, p.xi, p.x2, S);
+#pragma unroll
+  for (int k = 0; k < 5; k++)
+    r[k] = fma_(k == 0 || k == 3 ? T(0.5) : T(0.25), S[k], fma_(p.Gamma, h[k], T(-0.5) * adv[k]));
 }
 
 // Right-hand side of Eq. 1 at one cell,

@@ -138,105 +138,30 @@ __device__ __forceinline__ void cell_stencil(const double* __restrict__ p, int64
   }
 }
 
-// H of Eq. 3 from q and the neighbour sums s (the Laplacian's centre term is
-// in c.A1).  Q Q of a traceless Q: (QQ)_xy = c e - b f, (QQ)_xz = b e - c d,
-// (QQ)_yz = b c - a e with f = Qzz.
-__host__ __device__ __forceinline__ void cell_field(const double q[5], const double s[5], const CellPar& c,
-                                           double h[5]) {
-  const double a = q[0], b = q[1], cc = q[2], d = q[3], e = q[4], f = -(a + d);
-  const double b2 = b * b, c2 = cc * cc, e2 = e * e;
-  const double q0 = fma(a, a, b2 + c2), q3 = fma(d, d, b2 + e2), q5 = fma(f, f, c2 + e2);
-  const double q1 = fma(cc, e, -(b * f)), q2 = fma(b, e, -(cc * d)), q4 = fma(b, cc, -(a * e));
-  const double tr2 = (q0 + q3) + q5;
-  const double c1 = fma(-c.Ag, tr2, c.A1), c3 = c.Ag3 * tr2;
-  h[0] = fma(c1, a, fma(c.Ag, q0, fma(c.Kg, s[0], c3)));
-  h[1] = fma(c1, b, fma(c.Ag, q1, c.Kg * s[1]));
-  h[2] = fma(c1, cc, fma(c.Ag, q2, c.Kg * s[2]));
-  h[3] = fma(c1, d, fma(c.Ag, q3, fma(c.Kg, s[3], c3)));
-  h[4] = fma(c1, e, fma(c.Ag, q4, c.Kg * s[4]));
+// H of Eq. 3 from q and the neighbour sums s
+__host__ __device__ __forceinline__ void cell_field(const double q[5], const double s[5],
+                                                    const CellPar& c, double h[5]) {
+  molecular_field_tl(q, s, c.A1, c.Ag, c.Ag3, c.Kg, h);
 }
 
-// Eq. 5 without P0 (see physics.cuh: stress), times gs/2, from the plain
-// differences d[g][k].  d_aQ : d_bQ = 2 sum_k A_k B'_k with B'_0 = B_0 + B_3/2,
-// B'_3 = B_3 + B_0/2, B'_k = B_k otherwise.
+// Eq. 5 without P0, times gs/2, from the plain differences d[a][k]
 template <int DIM>
 __host__ __device__ __forceinline__ void cell_stress(const double q[5], const double h[5],
-                                            const double d[3][5], const CellPar& c,
-                                            double P[3][3]) {
-  const double Q[3][3] = {{q[0], q[1], q[2]}, {q[1], q[3], q[4]}, {q[2], q[4], -(q[0] + q[3])}};
-  const double H[3][3] = {{h[0], h[1], h[2]}, {h[1], h[3], h[4]}, {h[2], h[4], -(h[0] + h[3])}};
-  double X[3][3];
-#pragma unroll
-  for (int a = 0; a < 3; a++)
-#pragma unroll
-    for (int b = 0; b < 3; b++)
-      if ((a < DIM && b < DIM) || (a == 2 && b == 2))
-        X[a][b] = fma(Q[a][0], H[0][b], fma(Q[a][1], H[1][b], Q[a][2] * H[2][b]));
-  const double xq = c.s2 * ((X[0][0] + X[1][1]) + X[2][2]);
-  const double xq3 = xq * (1.0 / 3.0);
-#pragma unroll
-  for (int b = 0; b < DIM; b++) {
-    const double B0 = fma(0.5, d[b][3], d[b][0]), B3 = fma(0.5, d[b][0], d[b][3]);
-#pragma unroll
-    for (int a = 0; a <= b; a++) {
-      const double el =
-          fma(d[a][0], B0,
-              fma(d[a][3], B3,
-                  fma(d[a][1], d[b][1], fma(d[a][2], d[b][2], d[a][4] * d[b][4]))));
-      if (a == b) {
-        const double t = fma(xq, Q[a][a], fma(-c.s23, H[a][a], fma(-c.sK, el, xq3)));
-        P[a][a] = fma(-c.s2, X[a][a], t);
-      } else {
-        const double t = fma(xq, Q[a][b], fma(-c.s23, H[a][b], -(c.sK * el)));
-        P[a][b] = fma(-c.sm, X[a][b], fma(-c.sp, X[b][a], t));
-        P[b][a] = fma(-c.sm, X[b][a], fma(-c.sp, X[a][b], t));
-      }
-    }
-  }
+                                                     const double d[3][5], const CellPar& c,
+                                                     double P[3][3]) {
+  stress_tl<double, DIM>(q, h, d, c.s2, c.s23, c.sm, c.sp, c.sK, P);
 }
 
-// r = base + R of Eq. 1 with its trace projected out (see physics.cuh:
-// be_rhs_adv), from q, h = H, the plain differences d of Q and g[a][b] of u_a
-// along b, and u.  With N = 4/gs (xi D + W): N_aa = 2 xi g_aa,
-// N_ab = xi p + m, N_ba = xi p - m, p, m = g_ab +- g_ba.
+// r = base + R of Eq. 1 with its trace projected out, from q, h = H, u and the
+// plain differences d of Q and g[a][b] of u_a along b
 template <int DIM>
 __host__ __device__ __forceinline__ void cell_rhs(const double q[5], const double h[5],
-                                         const double d[3][5], const double u[3],
-                                         const double g[3][3], const CellPar& c,
-                                         const double base[5], double r[5]) {
+                                                  const double d[3][5], const double u[3],
+                                                  const double g[3][3], const CellPar& c,
+                                                  const double base[5], double r[5]) {
   constexpr bool D3 = DIM == 3;
-  const double third = 1.0 / 3.0;
-  const double t00 = q[0] + third, t11 = q[3] + third, t22 = third - (q[0] + q[3]);
-  const double b = q[1], cc = q[2], e = q[4];
-  const double n00 = c.x2 * g[0][0], n11 = c.x2 * g[1][1], n22 = D3 ? c.x2 * g[2][2] : 0.0;
-  const double p01 = g[0][1] + g[1][0], m01 = g[0][1] - g[1][0];
-  const double N01 = fma(c.xi, p01, m01), N10 = fma(c.xi, p01, -m01);
-  double N02 = 0.0, N20 = 0.0, N12 = 0.0, N21 = 0.0, off = b * p01;
-  if constexpr (D3) {
-    const double p02 = g[0][2] + g[2][0], m02 = g[0][2] - g[2][0];
-    const double p12 = g[1][2] + g[2][1], m12 = g[1][2] - g[2][1];
-    N02 = fma(c.xi, p02, m02), N20 = fma(c.xi, p02, -m02);
-    N12 = fma(c.xi, p12, m12), N21 = fma(c.xi, p12, -m12);
-    off = fma(cc, p02, fma(e, p12, off));
-  }
-  // 2 xi Q:G^T over gs/2, and the trace 2 xi div u / 3 over gs/2
-  const double tau = fma(q[0], D3 ? n00 - n22 : n00, fma(q[3], D3 ? n11 - n22 : n11, c.x2 * off));
-  const double tr = (D3 ? (n00 + n11) + n22 : n00 + n11) * (-1.0 / 9.0);
-  const double a0 = n00 - tau, a1 = n11 - tau, a2 = D3 ? n22 - tau : -tau;
   double S[5];
-  S[0] = fma(a0, t00, fma(N01, b, tr));
-  S[3] = fma(a1, t11, fma(N10, b, tr));
-  S[1] = fma(a0 + a1, b, fma(N01, t11, N10 * t00));
-  if constexpr (D3) {
-    S[0] = fma(N02, cc, S[0]);
-    S[3] = fma(N12, e, S[3]);
-    S[1] = fma(N02, e, fma(N12, cc, S[1]));
-    S[2] = fma(a0 + a2, cc, fma(N01, e, fma(N02, t22, fma(N20, t00, N21 * b))));
-    S[4] = fma(a1 + a2, e, fma(N10, cc, fma(N12, t22, fma(N20, b, N21 * t11))));
-  } else {
-    S[2] = fma(a0 + a2, cc, N01 * e);
-    S[4] = fma(a1 + a2, e, N10 * cc);
-  }
+  corotation_tl<double, DIM>(q, g, c.xi, c.x2, S);
   const double u0 = c.hu * u[0], u1 = c.hu * u[1], u2 = D3 ? c.hu * u[2] : 0.0;
 #pragma unroll
   for (int k = 0; k < 5; k++) {

@@ -186,9 +186,7 @@ __device__ __forceinline__ void lattice_stencil(const At& at, T v, T d2[3], T& l
 
 // stress on the ring-region cell of ring-phase thread t of a plane whose Q
 // box is in sq (z neighbours in sqm, sqp), into the Pi slot sp.  The first
-// derivatives are kept as plain differences (twice the central difference);
-// the stress sees them with K/4, which gives K dQ:dQ exactly (scalings by
-// powers of two are exact).
+// derivatives are kept as plain differences (twice the central difference).
 template <class Lat, class T, bool ISO>
 __device__ __forceinline__ void stress_ring_cell(int t, const T* __restrict__ sq,
                                                  const T* __restrict__ sqm,
@@ -199,32 +197,33 @@ __device__ __forceinline__ void stress_ring_cell(int t, const T* __restrict__ sq
   ring_cell(t, cx, cy, c);
   const int o = box_at(cx, cy);
   T q[5], dq2[3][5], lap[5], h[5], P[3][3];
-  // FP32: components (0, 1) and (2, 3) as packed pairs (same operations in
-  // the same order as the scalar form, lane by lane)
+  // FP32: components (0, 3) and (1, 2) as packed pairs (same operations in
+  // the same order as the scalar form, lane by lane), the pairs of dot5
   constexpr int KP = (std::is_same<T, float>::value && !ISO) ? 4 : 0;
   if constexpr (KP == 4) {
 #pragma unroll
-    for (int k = 0; k < 4; k += 2) {
+    for (int k = 0; k < 2; k++) {
+      const int j = 3 - k;
       const float* F0 = sq + k * BA;
-      const float* F1 = F0 + BA;
+      const float* F1 = sq + j * BA;
       const float2 v = pk(F0[o], F1[o]);
       const float2 xp = pk(F0[o + 1], F1[o + 1]), xm = pk(F0[o - 1], F1[o - 1]);
       const float2 yp = pk(F0[o + BXW], F1[o + BXW]), ym = pk(F0[o - BXW], F1[o - BXW]);
       float2 sum = padd(padd(xp, xm), padd(yp, ym));
       float2 dz = bc(0.0f);
       if (DIM == 3) {
-        const float2 zp = pk(sqp[k * BA + o], sqp[(k + 1) * BA + o]);
-        const float2 zm = pk(sqm[k * BA + o], sqm[(k + 1) * BA + o]);
+        const float2 zp = pk(sqp[k * BA + o], sqp[j * BA + o]);
+        const float2 zm = pk(sqm[k * BA + o], sqm[j * BA + o]);
         sum = padd(sum, padd(zp, zm));
         dz = psub(zp, zm);
       }
       const float2 dx = psub(xp, xm), dy = psub(yp, ym);
       const float2 l = pfma(bc(-2.0f * DIM), v, sum);
-      q[k] = v.x, q[k + 1] = v.y;
-      dq2[0][k] = dx.x, dq2[0][k + 1] = dx.y;
-      dq2[1][k] = dy.x, dq2[1][k + 1] = dy.y;
-      dq2[2][k] = dz.x, dq2[2][k + 1] = dz.y;
-      lap[k] = l.x, lap[k + 1] = l.y;
+      q[k] = v.x, q[j] = v.y;
+      dq2[0][k] = dx.x, dq2[0][j] = dx.y;
+      dq2[1][k] = dy.x, dq2[1][j] = dy.y;
+      dq2[2][k] = dz.x, dq2[2][j] = dz.y;
+      lap[k] = l.x, lap[j] = l.y;
     }
   }
 #pragma unroll
@@ -257,10 +256,8 @@ __device__ __forceinline__ void stress_ring_cell(int t, const T* __restrict__ sq
     dq2[2][k] = zp - zm;
     lap[k] = lap_points<T, DIM>(v, xp, xm, yp, ym, zp, zm);
   }
-  molecular_field(q, lap, p, h);
-  Par<T> p4 = p;
-  p4.K = p.K * T(0.25);
-  stress<T, DIM>(q, h, dq2, p4, P);
+  molecular_field_tl(q, lap, p.A1, p.Ag, p.Ag3, p.K, h);
+  stress_tl<T, DIM>(q, h, dq2, p.x2, p.x23, p.xm1, p.xp1, p.K * T(0.5), P);
 #pragma unroll
   for (int a = 0; a < DIM; a++)
 #pragma unroll
@@ -895,13 +892,6 @@ __device__ __forceinline__ bool fused_be_tile(const TileRef tile,
   const InstDev<T, G>& I = insts[tile.inst];
   const Dims d = I.d;
   const Par<T> p = I.p;
-  // the factors of Eq. 1 that multiply the velocity gradient, halved: the
-  // gradient arrives doubled (box_ugrad)
-  Par<T> p2 = p;
-  p2.hp = p.hp * T(0.5);
-  p2.hm = p.hm * T(0.5);
-  p2.x2 = p.x2 * T(0.5);
-  p2.x29 = p.x29 * T(0.5);
   const Field<T> Qout = I.q[cur ^ 1];
   const int zoff = Qout.L.zoff;
   const CUtensorMap* qmap = &qmaps[2 * tile.inst + cur];
@@ -956,7 +946,7 @@ __device__ __forceinline__ bool fused_be_tile(const TileRef tile,
     T q[5], adv[5], lap[5], u[3], G2[3][3], r[5];
     box_ugrad<Lat, T, ISO>(sU(su), sU(sum), sU(sup), o, u, G2);
     stencil_adv<Lat, T, ISO>(sQ(sq), sQ(sqm), sQ(sqp), o, BXW, BA, u, q, adv, lap);
-    be_rhs_adv<T>(q, adv, lap, G2, p2, r, T(-0.5));
+    be_rhs_tl<T, DIM>(q, adv, lap, G2, p, r);
     T* qpo = sQP(spo);
     if constexpr (std::is_same<T, float>::value) {
       // components (0, 1) and (2, 3) as packed pairs
@@ -992,7 +982,7 @@ __device__ __forceinline__ bool fused_be_tile(const TileRef tile,
     T qp[5], adv[5], lap[5], u[3], G2[3][3], r2[5];
     box_ugrad<Lat, T, ISO>(sU(su), sU(sum), sU(sup), o2, u, G2);
     stencil_adv<Lat, T, ISO>(sQP(sp), sQP(spm), sQP(spp), ic, RX1, A1, u, qp, adv, lap);
-    be_rhs_adv<T>(qp, adv, lap, G2, p2, r2, T(-0.5));
+    be_rhs_tl<T, DIM>(qp, adv, lap, G2, p, r2);
     // Q^{n+1} = Q^n + [R(Q^n) + R(Q^P)]/2 = [Q^n + Q^P + R(Q^P)]/2, since
     // Q^P = Q^n + R(Q^n)
     const T* qn = sQ(sq);

@@ -80,7 +80,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
 // kernel before it in the stream is still running.  grid_dep_wait() returns
 // once that kernel has completed and its memory operations are visible to
 // this grid (at once for a kernel launched without the attribute), so every
-// thread calls it before its first global access; grid_dep_trigger() allows
+// thread calls it before its first access to memory that kernels write;
+// grid_dep_trigger() allows
 // the next such kernel to be scheduled as soon as every block of this grid
 // has called it or exited (the implicit point without it).
 __device__ __forceinline__ void grid_dep_wait() {
@@ -88,6 +89,11 @@ __device__ __forceinline__ void grid_dep_wait() {
 }
 __device__ __forceinline__ void grid_dep_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// fetches a tensor map ahead of the first copy that uses it
+__device__ __forceinline__ void tma_prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
 
 // 4D tiled TMA load of one box into shared memory, completing on bar

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <vector>
 
 #include "adjoint.cuh"
@@ -104,7 +105,7 @@ struct InstHost {
   int obs_tz = 0;            // chunk list the obs_tiles were built for
   bool obs_taper = false;
   double* obs_part = nullptr;
-  double* prof = nullptr;
+  double* res = nullptr;  // observables: slot totals, S profile, error word
   int obs_blocks = 1;
   // adjoint work arrays (dense [comp][n])
   T* lQ[2] = {nullptr, nullptr};
@@ -148,6 +149,7 @@ class Engine final : public EngineBase {
     for (cudaEvent_t e : seg_ev_)
       if (e) cudaEventDestroy(e);
     for (void* ptr : allocs_) cudaFree(ptr);
+    free_host_words();
   }
 
   nlc_status init() {
@@ -591,8 +593,10 @@ class Engine final : public EngineBase {
         qs, nullptr, nullptr, I.q[cur_], I.g[cur_], I.d, args_.params[i].rho0, bad_);
     NLC_CK_LAUNCH("k_set_fields");
     unsigned long long nbad = 0;
-    NLC_CK(cudaMemcpyAsync(&nbad, bad_, sizeof(nbad), cudaMemcpyDeviceToHost, st));
+    void* hw = host_words(1);
+    NLC_CK(cudaMemcpyAsync(hw ? hw : &nbad, bad_, sizeof(nbad), cudaMemcpyDeviceToHost, st));
     NLC_CK(cudaStreamSynchronize(st));
+    if (hw) std::memcpy(&nbad, hw, sizeof(nbad));
     if (nbad) {
       err = "nlc_set_fields_f32: " + std::to_string(nbad) + " non-finite input values";
       return NLC_EUNSTABLE;
@@ -627,8 +631,10 @@ class Engine final : public EngineBase {
                                                    args_.params[i].rho0, bad_);
     NLC_CK_LAUNCH("k_set_fields");
     unsigned long long nbad = 0;
-    NLC_CK(cudaMemcpyAsync(&nbad, bad_, sizeof(nbad), cudaMemcpyDeviceToHost, st));
+    void* hw = host_words(1);
+    NLC_CK(cudaMemcpyAsync(hw ? hw : &nbad, bad_, sizeof(nbad), cudaMemcpyDeviceToHost, st));
     NLC_CK(cudaStreamSynchronize(st));
+    if (hw) std::memcpy(&nbad, hw, sizeof(nbad));
     if (nbad) {
       err = "nlc_set_fields: " + std::to_string(nbad) +
             " non-finite (or non-positive density) input values";
@@ -655,8 +661,7 @@ class Engine final : public EngineBase {
       if (u)
         NLC_CK(cudaMemcpyAsync(u, I.stage + 6 * n, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, st));
     }
-    NLC_CK(cudaStreamSynchronize(st));
-    return device_error();
+    return sync_and_check();
   }
 
   nlc_status get_populations(int i, double* f) override {
@@ -671,8 +676,7 @@ class Engine final : public EngineBase {
                                                          I.fstage);
     NLC_CK_LAUNCH("k_populations_out");
     NLC_CK(cudaMemcpyAsync(f, I.fstage, sizeof(double) * Q * n, cudaMemcpyDeviceToHost, st));
-    NLC_CK(cudaStreamSynchronize(st));
-    return device_error();
+    return sync_and_check();
   }
 
   size_t state_bytes() const override {
@@ -695,8 +699,7 @@ class Engine final : public EngineBase {
       NLC_CK(cudaMemcpyAsync(out, I.raw, sizeof(T) * 5 * n, cudaMemcpyDeviceToHost, st));
       out += sizeof(T) * 5 * n;
     }
-    NLC_CK(cudaStreamSynchronize(st));
-    return device_error();
+    return sync_and_check();
   }
 
   nlc_status load_state(const void* src) override {
@@ -828,7 +831,8 @@ class Engine final : public EngineBase {
     const Dims& d = I.d;
     cudaStream_t st = args_.stream;
     const double s_ref = 1.0 / 3.0;
-    const double* total = nullptr;
+    const double* partial = nullptr;
+    int nblocks = 0;
     if (!kCell && maps_ok_ && !iso_ && ix32_) {
       if constexpr (!kCell) {
       // one pass of the fused lb kernel in its observing form over this
@@ -864,10 +868,8 @@ class Engine final : public EngineBase {
         err = std::string("fused observables kernel: ") + cudaGetErrorString(e);
         return NLC_ECUDA;
       }
-      k_obs_final<<<OBS_SLOTS, 256, 0, st>>>(I.obs_part, I.obs_ntiles,
-                                             I.obs_part + (int64_t)I.obs_ntiles * OBS_SLOTS);
-      NLC_CK_LAUNCH("k_obs_final");
-      total = I.obs_part + (int64_t)I.obs_ntiles * OBS_SLOTS;
+      partial = I.obs_part;
+      nblocks = I.obs_ntiles;
       }
     } else {
       // stress of the current Q, then rho, u and the observables in one pass
@@ -876,10 +878,8 @@ class Engine final : public EngineBase {
       k_obs_state<Lat, T><<<I.obs_blocks, 256, 0, st>>>(I.q[cur_], I.g[cur_], I.pi, d, I.p,
                                                         s_ref, iso_, I.partial);
       NLC_CK_LAUNCH("k_obs_state");
-      k_obs_final<<<OBS_SLOTS, 256, 0, st>>>(I.partial, I.obs_blocks,
-                                             I.partial + I.obs_blocks * OBS_SLOTS);
-      NLC_CK_LAUNCH("k_obs_final");
-      total = I.partial + I.obs_blocks * OBS_SLOTS;
+      partial = I.partial;
+      nblocks = I.obs_blocks;
     }
     const int64_t rows = (int64_t)d.ny * d.nz;
     const int rows_per_chunk = profile_rows_per_chunk(d);
@@ -887,15 +887,20 @@ class Engine final : public EngineBase {
     dim3 pg((d.nx + 127) / 128, nchunks);
     k_profile_partial<T><<<pg, 128, 0, st>>>(I.q[cur_], d, rows_per_chunk, I.prof_partial);
     NLC_CK_LAUNCH("k_profile_partial");
-    k_profile_final<<<d.nx, 256, 0, st>>>(I.prof_partial, nchunks, d, I.prof);
-    NLC_CK_LAUNCH("k_profile_final");
-    double tot[OBS_SLOTS];
-    std::vector<double> prof(d.nx);
-    NLC_CK(cudaMemcpyAsync(tot, total, sizeof(tot), cudaMemcpyDeviceToHost, st));
-    NLC_CK(cudaMemcpyAsync(prof.data(), I.prof, sizeof(double) * d.nx, cudaMemcpyDeviceToHost, st));
+    k_obs_results<<<OBS_SLOTS + d.nx, 256, 0, st>>>(partial, nblocks, I.prof_partial, nchunks, d,
+                                                    derr_, I.res);
+    NLC_CK_LAUNCH("k_obs_results");
+    const size_t nres = OBS_SLOTS + (size_t)d.nx + 1;
+    double* res = host_words(nres);
+    if (!res) {
+      err = "no host memory for the observables";
+      return NLC_ENOMEM;
+    }
+    NLC_CK(cudaMemcpyAsync(res, I.res, sizeof(double) * nres, cudaMemcpyDeviceToHost, st));
     NLC_CK(cudaStreamSynchronize(st));
-    if ((s = device_error())) return s;
-    obs_from_totals(tot, prof.data(), d.nx, DIM == 2 || d.nz == 1, s_ref, out);
+    if (res[nres - 1] != 0.0 && (s = device_error())) return s;
+    const double *tot = res, *prof = res + OBS_SLOTS;
+    obs_from_totals(tot, prof, d.nx, DIM == 2 || d.nz == 1, s_ref, out);
     if (s_profile)
       for (int x = 0; x < d.nx; x++) s_profile[x] = prof[x];
     return NLC_OK;
@@ -925,6 +930,47 @@ class Engine final : public EngineBase {
     allocs_.push_back(ptr);
     *p = (U*)ptr;
     return NLC_OK;
+  }
+
+  // page-locked host words for small results (one copy, no staging by the
+  // driver); plain memory where none can be locked.  Kept by the engine and
+  // grown to the largest request.
+  double* host_words(size_t n) {
+    if (n <= hwords_n_) return hwords_;
+    free_host_words();
+    n = std::max<size_t>(n, 512);
+    if (cudaMallocHost((void**)&hwords_, sizeof(double) * n) == cudaSuccess) {
+      hwords_locked_ = true;
+    } else {
+      cudaGetLastError();
+      hwords_ = (double*)std::malloc(sizeof(double) * n);
+    }
+    hwords_n_ = hwords_ ? n : 0;
+    return hwords_;
+  }
+
+  void free_host_words() {
+    if (hwords_locked_)
+      cudaFreeHost(hwords_);
+    else
+      std::free(hwords_);
+    hwords_ = nullptr;
+    hwords_n_ = 0;
+    hwords_locked_ = false;
+  }
+
+  // waits for the stream and reports the device-side error word, which is
+  // read with the last copy before the wait
+  nlc_status sync_and_check() {
+    cudaStream_t st = args_.stream;
+    unsigned* w = (unsigned*)host_words(1);
+    if (w) {
+      NLC_CK(cudaMemcpyAsync(w, derr_, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+      NLC_CK(cudaStreamSynchronize(st));
+      return *w == DEV_ERR_NONE ? NLC_OK : device_error();
+    }
+    NLC_CK(cudaStreamSynchronize(st));
+    return device_error();
   }
 
   // device-side error word (bounded waits that ran out); read after a
@@ -1068,7 +1114,7 @@ class Engine final : public EngineBase {
     const int rpc = profile_rows_per_chunk(I.d);
     const int64_t nchunks = (rows + rpc - 1) / rpc;
     if ((s = alloc(&I.prof_partial, (size_t)(nchunks * I.d.nx)))) return s;
-    if ((s = alloc(&I.prof, (size_t)I.d.nx))) return s;
+    if ((s = alloc(&I.res, OBS_SLOTS + (size_t)I.d.nx + 1))) return s;
     return NLC_OK;
   }
 
@@ -1464,6 +1510,9 @@ class Engine final : public EngineBase {
   bool taper_ = false;  // tapered chunk lists (chunk_bounds)
   int ntiles_ = 0;
   bool maps_ok_ = false;
+  double* hwords_ = nullptr;  // host_words
+  size_t hwords_n_ = 0;
+  bool hwords_locked_ = false;
   // float64 arithmetic: descriptors of the cell kernels (ensure_cells)
   CellInst<G>* cells_dev_ = nullptr;
   double* cell_mrt_ = nullptr;   // [lattices][Q]

@@ -698,8 +698,7 @@ __device__ __forceinline__ bool fused_lb_tile(const TileRef tile,
     if (tid < NT) cell_plane(z1 - 1);
   }
   if constexpr (OBS) {
-    __shared__ double s_obs[32];
-    obs_block_out<T>(oacc, onbad, oumax, s_obs, obs_partial);
+    obs_block_out<T>(oacc, onbad, oumax, obs_partial);
   }
   // every copy issued was waited on: retire the barriers, so that the
   // block's next tile (persistent kernel) can initialise them again

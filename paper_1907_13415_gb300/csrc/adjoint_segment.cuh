@@ -20,6 +20,7 @@
 // steps the thread handles (a fixed cell-to-thread map, so the order is
 // fixed), then reduced per block in a fixed order into acc[block][3].
 #pragma once
+#include "convert.cuh"
 #include "adjoint.cuh"
 #include "common.cuh"
 #include "grid_sync.cuh"
@@ -103,9 +104,9 @@ __global__ void __launch_bounds__(SEG_THREADS) k_seg_reverse(SegArgs<T> a) {
   unsigned gen = 0;
   double acc3[3] = {0.0, 0.0, 0.0};
   auto take = [&](const ParBar<T>& pb) {
-    acc3[0] += (double)pb.gamma;
-    acc3[1] += (double)pb.K;
-    acc3[2] += (double)pb.Gamma;
+    acc3[0] += widen(pb.gamma);
+    acc3[1] += widen(pb.K);
+    acc3[2] += widen(pb.Gamma);
   };
   int lc = a.lc0;
   bool ok = true;

@@ -21,6 +21,9 @@
 #pragma once
 #include "adjoint.cuh"
 #include "adjoint_segment.cuh"
+#include "convert.cuh"
+#include "mrt.cuh"
+#include "step_fused.cuh"
 
 namespace nlc {
 
@@ -103,12 +106,15 @@ __global__ void __maxnreg__(96) k_seg_reverse_tiled(SegArgs<T> a, int tiles_x) {
   // Chebyshev distance from the tile (0 inside it)
   const int r = max(max(max(-lx, lx - (ATX - 1)), max(-ly, ly - (ATY - 1))), 0);
   const bool own = r == 0 && x0 + lx < d.nx && y0 + ly < d.ny;
+  // The parameter adjoints are summed in float64, which is slow on GB300; the
+  // stages leave their terms in shared memory and the sums are formed while
+  // the block waits at the grid barrier.  The terms sit in arrays that are
+  // free at the time (dq until stage 4, then qp, ua and gv): with arrays of
+  // their own the block would not fit beside a record block (16.9 KB) in the
+  // 64 KB of shared memory that the SM then sets aside, and the two kernels
+  // would run one after the other (2000 steps on 128^2: 37.6 instead of 28.0 ms;
+  // 32.7 ms with the sums in the stages).
   double acc3[3] = {0.0, 0.0, 0.0};
-  auto take = [&](const ParBar<T>& pb) {
-    acc3[0] += (double)pb.gamma;
-    acc3[1] += (double)pb.K;
-    acc3[2] += (double)pb.Gamma;
-  };
   unsigned gen = 0;
   int lc = a.lc0;
   bool ok = true;
@@ -138,7 +144,7 @@ __global__ void __maxnreg__(96) k_seg_reverse_tiled(SegArgs<T> a, int tiles_x) {
 #pragma unroll
         for (int b = 0; b < DIM; b++) S.gv[c * DIM + b][t] = Gb[c][b];
       }
-      if (own) take(pb);
+      if (own) S.dq[0][t] = pb.gamma, S.dq[1][t] = pb.K, S.dq[2][t] = pb.Gamma;
     }
     __syncthreads();
     // 2. predictor evaluation (adj_be1_at)
@@ -160,7 +166,7 @@ __global__ void __maxnreg__(96) k_seg_reverse_tiled(SegArgs<T> a, int tiles_x) {
 #pragma unroll
         for (int b = 0; b < DIM; b++) S.gv[c * DIM + b][t] += Gb[c][b];
       }
-      if (own) take(pb);
+      if (own) S.dq[3][t] = pb.gamma, S.dq[4][t] = pb.K, S.dq[5][t] = pb.Gamma;
     }
     __syncthreads();
     // 3. lb update (adj_lb_at): the pulled-back population adjoints are
@@ -207,11 +213,17 @@ __global__ void __maxnreg__(96) k_seg_reverse_tiled(SegArgs<T> a, int tiles_x) {
         }
       T q[5], dq[3][5], lap[5], h[5];
       q_stencil<T, DIM>(Q, x, y, 0, q, dq, lap);
-      molecular_field(q, lap, p, h);
+      molecular_field_tl(q, lap, p.A1, p.Ag, p.Ag3, p.K, h);
       T qb[5] = {}, hb[5] = {}, dqb[3][5] = {}, lapb[5] = {};
       ParBar<T> pb{T(0), T(0), T(0)};
       stress_vjp<T, DIM>(q, h, dq, p, Pib, qb, hb, dqb, pb);
       molecular_field_vjp(q, lap, p, hb, qb, lapb, pb);
+      if (own) {
+#pragma unroll
+        for (int k = 0; k < 5; k++) S.qp[k][t] = S.dq[k][t];
+        S.ua[0][t] = S.dq[5][t];
+        S.ua[1][t] = pb.gamma, S.gv[0][t] = pb.K, S.gv[1][t] = pb.Gamma;
+      }
 #pragma unroll
       for (int k = 0; k < 5; k++) {
         lq[k] += qb[k];
@@ -219,7 +231,6 @@ __global__ void __maxnreg__(96) k_seg_reverse_tiled(SegArgs<T> a, int tiles_x) {
 #pragma unroll
         for (int g = 0; g < DIM; g++) S.dq[g * 5 + k][t] = dqb[g][k];
       }
-      if (own) take(pb);
     }
     __syncthreads();
     // 5. stencil transposes (adj_stencil_at) on the owned cells
@@ -238,7 +249,14 @@ __global__ void __maxnreg__(96) k_seg_reverse_tiled(SegArgs<T> a, int tiles_x) {
     }
     // the adjoints of step j's state are complete everywhere before the
     // next reverse step reads them around every tile
-    if (!(ok = grid_sync(a.bar, gen, a.err, a.wait_ns))) break;
+    grid_arrive(a.bar);
+    if (own) {
+      const T terms[9] = {S.qp[0][t], S.qp[1][t], S.qp[2][t], S.qp[3][t], S.qp[4][t],
+                          S.ua[0][t], S.ua[1][t], S.gv[0][t], S.gv[1][t]};
+#pragma unroll
+      for (int k = 0; k < 9; k++) acc3[k % 3] += widen(terms[k]);
+    }
+    if (!(ok = grid_wait(a.bar, gen, a.err, a.wait_ns))) break;
     lc ^= 1;
   }
   if (!ok) return;
@@ -287,31 +305,46 @@ __global__ void __maxnreg__(72) k_seg_record_tiled(SegArgs<T> a, int tiles_x) {
   const int64_t idx = cell_of(d, x, y, 0);
   const int r = max(max(max(-lx, lx - (ATX - 1)), max(-ly, ly - (ATY - 1))), 0);
   const bool own = r == 0 && x0 + lx < d.nx && y0 + ly < d.ny;
-  // u and its gradient (u_stencil) from the box
-  auto u_box = [&](T u[3], T G[3][3]) {
+  // u and its plain differences (twice the gradient) from the box
+  auto u_box = [&](T u[2], T G2[3][3]) {
 #pragma unroll
-    for (int c = 0; c < 3; c++) {
-      if (c < DIM) {
-        u[c] = S.u[c][t];
-        G[c][0] = (S.u[c][t + 1] - S.u[c][t - 1]) / T(2);
-        G[c][1] = (S.u[c][t + ABW] - S.u[c][t - ABW]) / T(2);
-        G[c][2] = T(0);
-      } else {
-        u[c] = T(0);
-        G[c][0] = G[c][1] = G[c][2] = T(0);
-      }
+    for (int c = 0; c < DIM; c++) {
+      u[c] = S.u[c][t];
+      G2[c][0] = S.u[c][t + 1] - S.u[c][t - 1];
+      G2[c][1] = S.u[c][t + ABW] - S.u[c][t - ABW];
     }
   };
+  // q, its plain differences along x and y and its Laplacian
+  auto q_box = [&](const auto& at, T q[5], T d[3][5], T lap[5]) {
+#pragma unroll
+    for (int k = 0; k < 5; k++) {
+      const T v = at(k, 0, 0), xp = at(k, 1, 0), xm = at(k, -1, 0), yp = at(k, 0, 1),
+              ym = at(k, 0, -1);
+      q[k] = v;
+      d[0][k] = xp - xm;
+      d[1][k] = yp - ym;
+      lap[k] = lap_points<T, 2>(v, xp, xm, yp, ym, T(0), T(0));
+    }
+  };
+  auto advect = [&](const T u[2], const T d[3][5], T adv[5]) {
+#pragma unroll
+    for (int k = 0; k < 5; k++) adv[k] = fma_(u[0], d[0][k], u[1] * d[1][k]);
+  };
+  constexpr int NP = (Lat::Q - 1) / 2;
+  const T keep = T(1) - p.inv_tau, w2 = T(1.0 / 36.0);
+  const T cC = w2 * p.inv_tau, cG = T(3) * w2 * p.guo;
   unsigned gen = 0;
   for (int j = 0; j < a.len; j++) {
     const Field<T> Q = R.q(j), U = R.u(j), QP = R.qp(j), Qn = R.q(j + 1);
     T r1[5];
     // 1. stress (stress_at)
     if (r <= 3) {
-      T q[5], dq[3][5], lap[5], h[5], P[3][3];
-      q_stencil<T, DIM>(Q, x, y, 0, q, dq, lap);
-      molecular_field(q, lap, p, h);
-      stress<T, DIM>(q, h, dq, p, P);
+      T q[5], d2[3][5], lap[5], h[5], P[3][3];
+      const T* qc = Q.base + Q.off(0, x, y, 0);
+      const int64_t sy = Q.L.nxp, comp = Q.L.comp;
+      q_box([&](int k, int dx, int dy) { return qc[k * comp + dy * sy + dx]; }, q, d2, lap);
+      molecular_field_tl(q, lap, p.A1, p.Ag, p.Ag3, p.K, h);
+      stress_tl<T, DIM>(q, h, d2, p.x2, p.x23, p.xm1, p.xp1, p.K * T(0.5), P);
 #pragma unroll
       for (int c = 0; c < DIM; c++)
 #pragma unroll
@@ -323,7 +356,7 @@ __global__ void __maxnreg__(72) k_seg_record_tiled(SegArgs<T> a, int tiles_x) {
     __syncthreads();
     // 2. lb update (lb_at, BGK)
     if (r <= 2) {
-      T F[3], g[Lat::Q], rho, u[3];
+      T F[3], g[Lat::Q], rho, drho, J[3], u[3], gi[NP], gj[NP];
 #pragma unroll
       for (int c = 0; c < 3; c++) {
         T s = T(0);
@@ -337,27 +370,40 @@ __global__ void __maxnreg__(72) k_seg_record_tiled(SegArgs<T> a, int tiles_x) {
         F[c] = s;
       }
       pull<Lat, T>(R.g(j), d, x, y, 0, g);
-      moments<Lat, T>(g, F, p, rho, u);
-      collide_bgk<Lat, T>(g, rho, u, F, p);
+#pragma unroll
+      for (int k = 0; k < NP; k++)
+        gi[k] = g[pair_first<Lat>(k)], gj[k] = g[Lat::opp(pair_first<Lat>(k))];
+      moments_groups<Lat, T>(g[0], gi, gj, F, p.rho0, rho, drho, J, u);
+      collide_bgk_groups<Lat, T>(g[0], gi, gj, rho, drho, u, F, keep, cC, T(3) * cC, T(3) * cG,
+                                 cG);
 #pragma unroll
       for (int c = 0; c < DIM; c++) S.u[c][t] = u[c];
       if (own) {
         T* gout = R.g(j + 1);
+        gout[idx] = g[0];
 #pragma unroll
-        for (int i = 0; i < Lat::Q; i++) gout[(int64_t)i * d.n + idx] = g[i];
+        for (int k = 0; k < NP; k++) {
+          const int i = pair_first<Lat>(k);
+          gout[(int64_t)i * d.n + idx] = gi[k];
+          gout[(int64_t)Lat::opp(i) * d.n + idx] = gj[k];
+        }
         store_with_images<T, DIM, DIM>(U, d, x, y, 0, u);
       }
     }
     __syncthreads();
-    // 3. predictor (predict_at)
+    // 3. predictor (predict_at); r1 keeps Q + Q^P for the corrector
     if (r <= 1) {
-      T q[5], dq[3][5], lap[5], u[3], G[3][3], qp[5];
-      q_stencil<T, DIM>(Q, x, y, 0, q, dq, lap);
-      u_box(u, G);
-      be_rhs<T, DIM>(q, dq, lap, u, G, p, r1);
+      T q[5], d2[3][5], lap[5], u[2], G2[3][3], adv[5], qp[5];
+      const T* qc = Q.base + Q.off(0, x, y, 0);
+      const int64_t sy = Q.L.nxp, comp = Q.L.comp;
+      q_box([&](int k, int dx, int dy) { return qc[k * comp + dy * sy + dx]; }, q, d2, lap);
+      u_box(u, G2);
+      advect(u, d2, adv);
+      be_rhs_tl<T, DIM>(q, adv, lap, G2, p, r1);
 #pragma unroll
       for (int k = 0; k < 5; k++) {
         qp[k] = q[k] + r1[k];
+        r1[k] = q[k] + qp[k];
         S.qp[k][t] = qp[k];
       }
       if (own) store_with_images<T, 5, DIM>(QP, d, x, y, 0, qp);
@@ -365,22 +411,13 @@ __global__ void __maxnreg__(72) k_seg_record_tiled(SegArgs<T> a, int tiles_x) {
     __syncthreads();
     // 4. corrector (correct_at) on the owned cells
     if (own) {
-      T qp[5], dq[3][5], lap[5], u[3], G[3][3], r2[5], out[5];
+      T qp[5], d2[3][5], lap[5], u[2], G2[3][3], adv[5], r2[5], out[5];
+      q_box([&](int k, int dx, int dy) { return S.qp[k][t + dx + dy * ABW]; }, qp, d2, lap);
+      u_box(u, G2);
+      advect(u, d2, adv);
+      be_rhs_tl<T, DIM>(qp, adv, lap, G2, p, r2);
 #pragma unroll
-      for (int k = 0; k < 5; k++) {
-        const T v = S.qp[k][t];
-        const T xp = S.qp[k][t + 1], xm = S.qp[k][t - 1];
-        const T yp = S.qp[k][t + ABW], ym = S.qp[k][t - ABW];
-        qp[k] = v;
-        dq[0][k] = (xp - xm) / T(2);
-        dq[1][k] = (yp - ym) / T(2);
-        dq[2][k] = T(0);
-        lap[k] = (xp + xm - T(2) * v) + (yp + ym - T(2) * v);
-      }
-      u_box(u, G);
-      be_rhs<T, DIM>(qp, dq, lap, u, G, p, r2);
-#pragma unroll
-      for (int k = 0; k < 5; k++) out[k] = Q.at(k, x, y, 0) + (r1[k] + r2[k]) / T(2);
+      for (int k = 0; k < 5; k++) out[k] = (r1[k] + r2[k]) * T(0.5);
       store_with_images<T, 5, DIM>(Qn, d, x, y, 0, out);
     }
     // the step's records are complete everywhere before the next step

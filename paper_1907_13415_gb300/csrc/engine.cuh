@@ -1193,7 +1193,12 @@ class Engine final : public EngineBase {
     if (!I.bar) {
       if ((s = alloc(&I.bar, 3))) return s;
       const int64_t want = (I.d.n + SEG_THREADS - 1) / SEG_THREADS;
-      I.seg_grid = (int)std::min<int64_t>(seg_grid_max(), want);
+      // as many blocks as are resident, or, when that takes several rounds
+      // over the cells, only as many as the rounds need: every block costs
+      // an arrival at each grid barrier
+      const int64_t fit = seg_grid_max();
+      const int64_t rounds = fit > 0 ? (want + fit - 1) / fit : 1;
+      I.seg_grid = (int)std::min<int64_t>(fit, (want + rounds - 1) / rounds);
       I.acc_slots = I.seg_grid;
       if ((s = plan_tiled_reverse(I))) return s;
     }

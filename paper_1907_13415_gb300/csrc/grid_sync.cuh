@@ -28,13 +28,18 @@ __device__ __forceinline__ void red_release_gpu_add(unsigned* p, unsigned v) {
 // is cumulative: generation g completes at (g + 1) gridDim.x).  The poll is
 // bounded by wait_ns nanoseconds of %globaltimer; returns false in every
 // thread of the block if it ran out.
-__device__ __forceinline__ bool grid_sync(GridBarrier* b, unsigned& gen, unsigned* err,
-                                          uint64_t wait_ns) {
+__device__ __forceinline__ void grid_arrive(GridBarrier* b) {
   __syncthreads();
+  if (threadIdx.x == 0) red_release_gpu_add(&b->arrived, 1u);
+}
+
+// the wait for the generation this block has arrived at; work of the block
+// that other blocks do not need can stand between the two
+__device__ __forceinline__ bool grid_wait(GridBarrier* b, unsigned& gen, unsigned* err,
+                                          uint64_t wait_ns) {
   int ok = 1;
   if (threadIdx.x == 0) {
     const unsigned target = (gen + 1) * gridDim.x;
-    red_release_gpu_add(&b->arrived, 1u);
     if (ld_acquire_gpu(&b->arrived) < target) {
       const uint64_t t0 = global_ns();
       while (ld_acquire_gpu(&b->arrived) < target) {
@@ -48,6 +53,12 @@ __device__ __forceinline__ bool grid_sync(GridBarrier* b, unsigned& gen, unsigne
   }
   gen++;
   return __syncthreads_and(ok) != 0;
+}
+
+__device__ __forceinline__ bool grid_sync(GridBarrier* b, unsigned& gen, unsigned* err,
+                                          uint64_t wait_ns) {
+  grid_arrive(b);
+  return grid_wait(b, gen, err, wait_ns);
 }
 
 // orders this thread's earlier generic-proxy global writes (made visible

@@ -1,7 +1,7 @@
-// mrt.cuh -- the multiple-relaxation-time collision of physics.cuh
-// (collide_mrt) on sums and differences of opposite populations.
+// mrt.cuh -- the collisions of physics.cuh (collide_bgk, collide_mrt) on sums
+// and differences of opposite populations.
 //
-// The moment rows are even or odd under c -> -c and built from few groups of
+// The moment rows of the multiple-relaxation-time collision are even or odd under c -> -c and built from few groups of
 // velocities: the even ones see only the sum of each axis pair, and the sum
 // and difference of the two pairs of each diagonal plane; the odd ones the
 // differences along one axis.  Transforming those groups instead of the
@@ -86,6 +86,54 @@ __host__ __device__ __forceinline__ void moments_groups(T g0, const T* gi, const
     inv = T(1) / rho;
 #pragma unroll
   for (int a = 0; a < Lat::DIM; a++) u[a] = fma_(T(0.5), F[a], J[a]) * inv;
+}
+
+// BGK collision with the source term (physics.cuh: collide_bgk) on the same
+// groups, over the diagonal weight w2: even part C + M_aa (+ M_bb +- M_ab), odd
+// part L_a (+- L_b) with t = A u + B F, M_aa = u_a t_a, M_ab = u_a t_b + u_b t_a
+// and L = R u + G F; the even part of the axis pairs (the rest population)
+// carries the weight ratio ra (r0).  cC = w2/tau, cR = 3 w2/tau, cB = 9 w2 k,
+// cG = 3 w2 k, k = 1 - 1/(2 tau), keep = 1 - 1/tau.
+template <class Lat, class T>
+__host__ __device__ __forceinline__ void collide_bgk_groups(T& g0, T* gi, T* gj, T rho, T drho,
+                                                            const T u[3], const T F[3], T keep,
+                                                            T cC, T cR, T cB, T cG) {
+  constexpr int DIM = Lat::DIM, NP = (Lat::Q - 1) / 2;
+  constexpr T ra = DIM == 2 ? T(4) : T(2), r0 = DIM == 2 ? T(16) : T(12);
+  const T R = cR * rho, A = T(1.5) * R;
+  T t[3], L[3], M[3], B[3];
+#pragma unroll
+  for (int a = 0; a < DIM; a++) {
+    t[a] = fma_(A, u[a], cB * F[a]);
+    L[a] = fma_(R, u[a], cG * F[a]);
+    M[a] = u[a] * t[a];
+  }
+  const T Ms = DIM == 3 ? (M[0] + M[1]) + M[2] : M[0] + M[1];
+  const T C = fma_(cC, drho, Ms * T(-1.0 / 3.0));
+  g0 = fma_(keep, g0, r0 * C);
+#pragma unroll
+  for (int a = 0; a < DIM; a++) B[a] = C + M[a];
+#pragma unroll
+  for (int k = 0; k < NP; k++) {
+    const int i = pair_first<Lat>(k);
+    int a = -1, b = -1;  // the axes the pair moves along
+#pragma unroll
+    for (int o = 0; o < DIM; o++)
+      if (Lat::c(i, o) != 0) (a < 0 ? a : b) = o;
+    if (b < 0) {
+      gi[k] = fma_(ra, B[a] + L[a], keep * gi[k]);
+      gj[k] = fma_(ra, B[a] - L[a], keep * gj[k]);
+    } else {
+      const bool same = Lat::c(i, a) == Lat::c(i, b);
+      const T Mab = fma_(u[a], t[b], u[b] * t[a]);
+      const T N = B[a] + M[b];
+      const T E = same ? N + Mab : N - Mab;
+      T O = same ? L[a] + L[b] : L[a] - L[b];  // odd part along c_i
+      if (Lat::c(i, a) < 0) O = -O;
+      gi[k] = fma_(keep, gi[k], E + O);
+      gj[k] = fma_(keep, gj[k], E - O);
+    }
+  }
 }
 
 // g0, gi, gj: the rest population and the opposite pairs (pair_first and its

@@ -273,57 +273,15 @@ __global__ void __launch_bounds__(CELL_T) k_cell_lb(const CellInst<G>* __restric
   double rho, drho, J[3], u[3];
   moments_groups<Lat, double>(g0, gi, gj, F, c.rho0, rho, drho, J, u);
   auto put = [&](int i, double v) { gout[i * d.n + idx] = store_as<G>(v); };
-  if (I->mrt) {
+  if (I->mrt)
     collide_mrt_groups<Lat, double>(g0, gi, gj, rho, drho, J, u, F, I->mrt);
-    put(0, g0);
+  else
+    collide_bgk_groups<Lat, double>(g0, gi, gj, rho, drho, u, F, c.keep, c.cC, c.cR, c.cB, c.cG);
+  put(0, g0);
 #pragma unroll
-    for (int k = 0; k < NP; k++) {
-      put(pair_first<Lat>(k), gi[k]);
-      put(Lat::opp(pair_first<Lat>(k)), gj[k]);
-    }
-  } else {
-    // BGK with the source term (physics.cuh: collide_bgk) over the diagonal
-    // weight w2: even part C + M_aa (+ M_bb +- M_ab), odd part L_a (+- L_b)
-    // with t = A u + B F, M_aa = u_a t_a, M_ab = u_a t_b + u_b t_a and
-    // L = R u + G F; the even part of the axis pairs (the rest population)
-    // carries the weight ratio ra (r0)
-    constexpr double ra = DIM == 2 ? 4.0 : 2.0, r0 = DIM == 2 ? 16.0 : 12.0;
-    const double R = c.cR * rho, A = 1.5 * R;
-    double t[3], L[3], M[3];
-#pragma unroll
-    for (int a = 0; a < DIM; a++) {
-      t[a] = fma(A, u[a], c.cB * F[a]);
-      L[a] = fma(R, u[a], c.cG * F[a]);
-      M[a] = u[a] * t[a];
-    }
-    const double Ms = DIM == 3 ? (M[0] + M[1]) + M[2] : M[0] + M[1];
-    const double C = fma(c.cC, drho, Ms * (-1.0 / 3.0));
-    put(0, fma(c.keep, g0, r0 * C));
-    double B[3];  // C + M_aa
-#pragma unroll
-    for (int a = 0; a < DIM; a++) B[a] = C + M[a];
-#pragma unroll
-    for (int k = 0; k < NP; k++) {
-      const int i = pair_first<Lat>(k), j = Lat::opp(i);
-      int a = -1, b = -1;  // the axes the pair moves along
-#pragma unroll
-      for (int o = 0; o < DIM; o++)
-        if (Lat::c(i, o) != 0) (a < 0 ? a : b) = o;
-      if (b < 0) {
-        put(i, fma(ra, B[a] + L[a], c.keep * gi[k]));
-        put(j, fma(ra, B[a] - L[a], c.keep * gj[k]));
-      } else {
-        const bool same = Lat::c(i, a) == Lat::c(i, b);
-        const double Mab = fma(u[a], t[b], u[b] * t[a]);
-        const double N = B[a] + M[b];
-        const double E = same ? N + Mab : N - Mab;
-        // odd part along c_i
-        double O = same ? L[a] + L[b] : L[a] - L[b];
-        if (Lat::c(i, a) < 0) O = -O;
-        put(i, fma(c.keep, gi[k], E + O));
-        put(j, fma(c.keep, gj[k], E - O));
-      }
-    }
+  for (int k = 0; k < NP; k++) {
+    put(pair_first<Lat>(k), gi[k]);
+    put(Lat::opp(pair_first<Lat>(k)), gj[k]);
   }
   const Field<double> U{I->u, I->L};
   store_with_images<double, DIM, DIM>(U, d, x, y, z, u);

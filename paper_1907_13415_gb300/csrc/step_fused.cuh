@@ -713,8 +713,9 @@ __device__ __forceinline__ bool fused_lb_tile(const TileRef tile,
 // kernel of the stream (launched with programmatic serialisation) may be
 // scheduled at once and wait for this one on the device; otherwise its
 // blocks would hold SM slots that this kernel's later waves need.
-template <class Lat, class T, class G, bool MRT, bool ISO, bool IX32, bool OBS = false>
-__global__ void __launch_bounds__(LbCfg<Lat, T>::THREADS, LbCfg<Lat, T>::MINB)
+template <class Lat, class T, class G, bool MRT, bool ISO, bool IX32, bool OBS = false,
+          int MINB = LbCfg<Lat, T>::MINB>
+__global__ void __launch_bounds__(LbCfg<Lat, T>::THREADS, MINB)
     k_fused_lb(const InstDev<T, G>* __restrict__ insts,
                const CUtensorMap* __restrict__ qmaps,
                const TileRef* __restrict__ tiles, int cur,
@@ -1087,8 +1088,8 @@ __device__ __forceinline__ bool fused_be_tile(const TileRef tile,
   return true;
 }
 
-template <class Lat, class T, class G, bool ISO>
-__global__ void __launch_bounds__(BeCfg<Lat, T>::THREADS, BeCfg<Lat, T>::MINB)
+template <class Lat, class T, class G, bool ISO, int MINB = BeCfg<Lat, T>::MINB>
+__global__ void __launch_bounds__(BeCfg<Lat, T>::THREADS, MINB)
     k_fused_be(const InstDev<T, G>* __restrict__ insts,
                const CUtensorMap* __restrict__ qmaps,
                const CUtensorMap* __restrict__ umaps,
@@ -1256,20 +1257,46 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int threads, s
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Blocks per SM that a step kernel of a launch of several waves is compiled
+// for.  On a single plane the float32 kernels fit in 56 registers without
+// spills and their shared memory in a third of an SM, so three blocks hide
+// more of each other's barrier waits than two with 72-80 registers; a launch
+// of one wave keeps the form for two, which has more loads in flight per
+// thread and, started early behind the previous kernel, spreads evenly.
+// us per step, two / three blocks (FP32): 64-lattice sweep 109.5 / 94.5,
+// 512^2 20.0 / 17.3, 2035 x 1501 138 / 126, 4096^2 643 / 611; 256^2 (256
+// blocks) 6.2 / 7.8.
+template <class Lat, class T>
+constexpr int many_blocks() {
+  return Lat::DIM == 2 && sizeof(T) == 4 ? 3 : 0;
+}
+
+// Launches kernel2, compiled for the default number of blocks per SM, or,
+// when the launch takes more than one wave of it, kernel3 (if given).
+template <class K2, class K3, class... Args>
+cudaError_t launch_step(K2 kernel2, K3 kernel3, bool have3, int threads, size_t smem, int ntiles,
+                        unsigned long long* configured, ResidentCache* resident, cudaStream_t st,
+                        Args... args) {
+  cudaError_t e = set_smem(kernel2, smem, &configured[0]);
+  if (e != cudaSuccess) return e;
+  const bool one_wave = ntiles <= resident_blocks(kernel2, threads, smem, *resident);
+  if (one_wave || !have3)
+    return launch_pdl(kernel2, ntiles, threads, smem, st, args..., one_wave ? 1 : 0);
+  if ((e = set_smem(kernel3, smem, &configured[1])) != cudaSuccess) return e;
+  return launch_pdl(kernel3, ntiles, threads, smem, st, args..., 0);
+}
+
 template <class Lat, class T, class G, bool MRT, bool ISO, bool IX32>
 cudaError_t launch_fused_lb_as(const InstDev<T, G>* insts, const CUtensorMap* qmaps,
                                const TileRef* tiles, int ntiles, int cur, unsigned* err,
                                cudaStream_t st) {
-  static unsigned long long configured = 0;
+  static unsigned long long configured[2] = {0, 0};
   static ResidentCache resident;
-  auto kernel = k_fused_lb<Lat, T, G, MRT, ISO, IX32>;
-  constexpr int threads = LbCfg<Lat, T>::THREADS;
-  constexpr size_t smem = LbCfg<Lat, T>::bytes;
-  cudaError_t e = set_smem(kernel, smem, &configured);
-  if (e != cudaSuccess) return e;
-  const int early = ntiles <= resident_blocks(kernel, threads, smem, resident) ? 1 : 0;
-  return launch_pdl(kernel, ntiles, threads, smem, st, insts, qmaps, tiles, cur, err,
-                    (double*)nullptr, early);
+  constexpr int M2 = LbCfg<Lat, T>::MINB, M3 = many_blocks<Lat, T>();
+  return launch_step(k_fused_lb<Lat, T, G, MRT, ISO, IX32, false, M2>,
+                     k_fused_lb<Lat, T, G, MRT, ISO, IX32, false, M3 ? M3 : M2>, M3 != 0,
+                     LbCfg<Lat, T>::THREADS, LbCfg<Lat, T>::bytes, ntiles, configured, &resident,
+                     st, insts, qmaps, tiles, cur, err, (double*)nullptr);
 }
 
 // the observables of the current state (buffers cur) over the tiles given
@@ -1316,16 +1343,12 @@ template <class Lat, class T, class G, bool ISO>
 cudaError_t launch_fused_be_as(const InstDev<T, G>* insts, const CUtensorMap* qmaps,
                                const CUtensorMap* umaps, const TileRef* tiles, int ntiles,
                                int cur, unsigned* err, cudaStream_t st) {
-  static unsigned long long configured = 0;
+  static unsigned long long configured[2] = {0, 0};
   static ResidentCache resident;
-  auto kernel = k_fused_be<Lat, T, G, ISO>;
-  constexpr int threads = BeCfg<Lat, T>::THREADS;
-  constexpr size_t smem = BeCfg<Lat, T>::bytes;
-  cudaError_t e = set_smem(kernel, smem, &configured);
-  if (e != cudaSuccess) return e;
-  const int early = ntiles <= resident_blocks(kernel, threads, smem, resident) ? 1 : 0;
-  return launch_pdl(kernel, ntiles, threads, smem, st, insts, qmaps, umaps, tiles, cur, err,
-                    early);
+  constexpr int M2 = BeCfg<Lat, T>::MINB, M3 = many_blocks<Lat, T>();
+  return launch_step(k_fused_be<Lat, T, G, ISO, M2>, k_fused_be<Lat, T, G, ISO, M3 ? M3 : M2>,
+                     M3 != 0, BeCfg<Lat, T>::THREADS, BeCfg<Lat, T>::bytes, ntiles, configured,
+                     &resident, st, insts, qmaps, umaps, tiles, cur, err);
 }
 
 template <class Lat, class T, class G>

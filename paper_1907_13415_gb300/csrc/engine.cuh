@@ -221,6 +221,16 @@ class Engine final : public EngineBase {
       InstHost<T, G>& I = inst_[i];
       I.tz = tz > 0 ? std::min(tz, column_length<Lat>(I.d))
                     : fused_tz<Lat>(I.d, (int64_t)tiles.size());
+      if (tz <= 0 && DIM == 3 && !kCell && inst_.size() == 1) {
+        // the estimate covers one float32 D3Q19 lattice with the device to
+        // itself (us per step at its depth / the rule above: 128^3 177 / 199,
+        // 160^3 319 / 326, 70 x 180 x 50 80 / 91, 32^3 16 / 24)
+        int dev = 0, sms = 0;
+        NLC_CK(cudaGetDevice(&dev));
+        NLC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        const long columns = (long)((I.d.nx + FTX - 1) / FTX) * ((I.d.ny + FTY - 1) / FTY);
+        I.tz = estimated_depth(I.d.nz, columns, sms, I.tz);
+      }
       append_tiles<Lat>((int)i, I.d, I.tz, taper_, &tiles);
     }
     NLC_CK(cudaStreamSynchronize(st));  // no step may still read the old list

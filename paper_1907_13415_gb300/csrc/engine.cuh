@@ -414,7 +414,7 @@ class Engine final : public EngineBase {
     any_mrt_ = false;
     for (bool b : mrt_on_) any_mrt_ = any_mrt_ || b;
     drop_graphs();
-    return NLC_OK;
+    return cells_dev_ ? ensure_cells() : NLC_OK;
   }
 
   void invalidate_graphs() override { drop_graphs(); }
@@ -437,7 +437,7 @@ class Engine final : public EngineBase {
       cells_stale_ = true;
     }
     iso_ = iso;
-    return NLC_OK;
+    return cells_dev_ ? ensure_cells() : NLC_OK;
   }
 
   nlc_status set_params(int i, const nlc_params& q) override {
@@ -587,7 +587,7 @@ class Engine final : public EngineBase {
   nlc_status set_fields_f32(int i, const float* Q5) override {
     InstHost<T, G>& I = inst_[i];
     nlc_status s;
-    if ((s = ensure_staging(I))) return s;
+    if ((s = ensure_staging(I)) || (s = ensure_cells())) return s;
     const int64_t n = I.d.n;
     cudaStream_t st = args_.stream;
     // device arrays are read in place too (a caller that uploads the next
@@ -618,7 +618,7 @@ class Engine final : public EngineBase {
                         const double* u) override {
     InstHost<T, G>& I = inst_[i];
     nlc_status s;
-    if ((s = ensure_staging(I))) return s;
+    if ((s = ensure_staging(I)) || (s = ensure_cells())) return s;
     const int64_t n = I.d.n;
     cudaStream_t st = args_.stream;
     // pinned inputs are read in place by the kernel (the transfer then
@@ -715,6 +715,7 @@ class Engine final : public EngineBase {
   nlc_status load_state(const void* src) override {
     cudaStream_t st = args_.stream;
     const char* in = (const char*)src;
+    if (nlc_status cs = ensure_cells()) return cs;
     for (auto& I : inst_) {
       nlc_status s;
       if (!I.raw && (s = alloc(&I.raw, (size_t)5 * I.d.n))) return s;
@@ -1031,6 +1032,12 @@ class Engine final : public EngineBase {
   nlc_status ensure_cells() {
     if constexpr (kCell) {
       if (cells_off_ || (cells_dev_ && !cells_stale_)) return NLC_OK;
+      // nothing may be allocated or waited for inside a caller's stream
+      // capture: such a step takes the tiled kernels (set_fields, load_state
+      // and the calls that change the descriptors build them beforehand)
+      cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+      NLC_CK(cudaStreamIsCapturing(args_.stream, &capturing));
+      if (capturing != cudaStreamCaptureStatusNone) return NLC_OK;
       nlc_status s;
       const size_t n = inst_.size();
       for (size_t i = 0; i < n; i++) {
@@ -1411,7 +1418,7 @@ class Engine final : public EngineBase {
 
   // one step of every lattice: two launches over the joint tile list
   nlc_status step_fused(cudaStream_t st) {
-    if (cells_dev_ && !cells_off_) return step_cells(st);
+    if (cells_dev_ && !cells_off_ && !cells_stale_) return step_cells(st);
     const int a = cur_;
     const int e0 = mark();
     cudaError_t e = launch_fused_lb<Lat, T>(insts_dev_, qmaps_dev_, tiles_dev_, ntiles_, a,

@@ -62,8 +62,8 @@ def alg_bytes(precision):
 # on; reported as null once those sources change.
 NCU_TRAFFIC = {
     # 256 x 256 x 64 capture (4,194,304 cells), see profiles/
-    "fused_lb": ((431.065600e6 + 333.152000e6) / 4194304, "967ef2352f20c314"),
-    "fused_be": ((155.785728e6 + 61.327104e6) / 4194304, "967ef2352f20c314"),
+    "fused_lb": ((431.478784e6 + 332.688640e6) / 4194304, "f597b7235c9f04e9"),
+    "fused_be": ((155.643904e6 + 57.826048e6) / 4194304, "f597b7235c9f04e9"),
 }
 
 KERNEL_SOURCES = ["paper_1907_13415_gb300/csrc/step_fused.cuh",
@@ -73,6 +73,8 @@ KERNEL_SOURCES = ["paper_1907_13415_gb300/csrc/step_fused.cuh",
                   "paper_1907_13415_gb300/csrc/common.cuh",
                   "paper_1907_13415_gb300/csrc/packed.cuh",
                   "paper_1907_13415_gb300/csrc/tma.cuh",
+                  "paper_1907_13415_gb300/csrc/mrt.cuh",
+                  "paper_1907_13415_gb300/csrc/convert.cuh",
                   "paper_1907_13415_gb300/csrc/aux_kernels.cuh"]
 
 

@@ -265,8 +265,9 @@ NLC_API nlc_status nlc_set_schedule(nlc_ctx* ctx, int32_t schedule);
  * remain, then chunks halving down to about 8 planes (tiles); the blocks run
  * chunk by chunk, so the last blocks are short and the last wave over the
  * SMs idles less of the GPU.  Neither changes any result: every chunk list
- * computes the same step bit for bit.  A runtime choice of this library;
- * the paper has no counterpart.  Synchronises the stream.  Errors:
+ * computes the same step bit for bit.  (The float64 kernels of nlc_step do
+ * not use the list.)  A runtime choice of this library; the paper has no
+ * counterpart.  Synchronises the stream.  Errors:
  * NLC_EINVAL (chunk < 0, taper not 0 or 1). */
 NLC_API nlc_status nlc_set_chunk(nlc_ctx* ctx, int32_t chunk, int32_t taper);
 
@@ -328,11 +329,15 @@ NLC_API nlc_status nlc_get_fields(nlc_ctx* ctx, int32_t inst, double* Q5,
 NLC_API nlc_status nlc_get_populations(nlc_ctx* ctx, int32_t inst, double* f);
 
 /* Advances every lattice of the context by n time steps (n >= 0).  Queued
- * on the context's stream; returns launch errors only.  The two kernels of
- * a step are launched with programmatic dependent launch: each may be
- * scheduled while the kernel before it in the stream (the caller's own,
- * too) is finishing, and waits on the device for that kernel to complete
- * before it touches memory, so stream order holds for every buffer. */
+ * on the context's stream; returns launch errors only.  A step is two tiled
+ * kernels, or, in float64 arithmetic (NLC_FP64, NLC_FP32_QF64), four kernels
+ * of one cell per thread, which take the workspaces of the unfused schedule
+ * (nlc_set_fields allocates them; where they do not fit the tiled kernels
+ * run).  The kernels are launched with programmatic dependent launch: each
+ * may be scheduled while the kernel before it in the stream (the caller's
+ * own, too) is finishing, and waits on the device for that kernel to
+ * complete before it touches memory that kernels write, so stream order
+ * holds for every buffer. */
 NLC_API nlc_status nlc_step(nlc_ctx* ctx, int64_t n);
 
 /* Computes the observables of the current state of instance inst into *out

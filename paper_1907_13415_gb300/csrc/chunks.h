@@ -52,6 +52,8 @@ inline double estimate_step_us(int nz, long columns, int tz, int sms) {
   const long blocks = columns * (long)(b.size() - 1);
   if (blocks <= sms) return 3.9 * (b[1] + extra);
   if (blocks <= 2L * sms) return 6.3 * (b[1] + extra);
+  if (blocks > 200L * sms)  // the last wave no longer matters
+    return 5.0 * columns * (nz + extra * (double)(b.size() - 1)) / (2.0 * sms);
   std::map<double, long> free_at;  // time -> slots free from then on
   free_at[0.0] = 2L * sms;
   for (size_t k = 0; k + 1 < b.size(); k++) {

@@ -715,7 +715,6 @@ class Engine final : public EngineBase {
   nlc_status load_state(const void* src) override {
     cudaStream_t st = args_.stream;
     const char* in = (const char*)src;
-    if (nlc_status cs = ensure_cells()) return cs;
     for (auto& I : inst_) {
       nlc_status s;
       if (!I.raw && (s = alloc(&I.raw, (size_t)5 * I.d.n))) return s;
@@ -729,7 +728,7 @@ class Engine final : public EngineBase {
     }
     NLC_CK(cudaStreamSynchronize(st));
     cur_ = 0;
-    return NLC_OK;
+    return ensure_cells();
   }
 
 
@@ -1035,8 +1034,13 @@ class Engine final : public EngineBase {
       // nothing may be allocated or waited for inside a caller's stream
       // capture: such a step takes the tiled kernels (set_fields, load_state
       // and the calls that change the descriptors build them beforehand)
+      // (the query itself fails on the legacy stream while another stream is
+      // being captured)
       cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-      NLC_CK(cudaStreamIsCapturing(args_.stream, &capturing));
+      if (cudaStreamIsCapturing(args_.stream, &capturing) != cudaSuccess) {
+        cudaGetLastError();
+        return NLC_OK;
+      }
       if (capturing != cudaStreamCaptureStatusNone) return NLC_OK;
       nlc_status s;
       const size_t n = inst_.size();

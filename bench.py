@@ -62,8 +62,8 @@ def alg_bytes(precision):
 # on; reported as null once those sources change.
 NCU_TRAFFIC = {
     # 256 x 256 x 64 capture (4,194,304 cells), see profiles/
-    "fused_lb": ((431.478784e6 + 332.688640e6) / 4194304, "f597b7235c9f04e9"),
-    "fused_be": ((155.643904e6 + 57.826048e6) / 4194304, "f597b7235c9f04e9"),
+    "fused_lb": ((431.041792e6 + 332.873216e6) / 4194304, "08c3b02cbcc4f468"),
+    "fused_be": ((155.696384e6 + 57.724160e6) / 4194304, "08c3b02cbcc4f468"),
 }
 
 KERNEL_SOURCES = ["paper_1907_13415_gb300/csrc/step_fused.cuh",

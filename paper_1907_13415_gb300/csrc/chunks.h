@@ -44,8 +44,9 @@ inline std::vector<int> chunk_bounds(int nz, int tz, bool taper) {
 // recomputes and its start) times 3.9 us when it has an SM to itself, 6.3 us
 // when one wave of blocks fills SMs twice (their phases coincide), 5.0 us in
 // several waves, where the blocks of a list start in order on the first free
-// slot.  Fitted to 13 lattices from 20 to 256 planes a side; among all uniform
-// depths its choice is within 1.4% of the fastest on average.
+// slot.  Fitted to 13 lattices from 20 to 256 planes a side: choosing among
+// uniform and tapered lists by it came within 1.4% of the fastest on average,
+// and up to 7% on one lattice.
 inline double estimate_step_us(int nz, long columns, int tz, int sms) {
   const double extra = 1.5;
   const std::vector<int> b = chunk_bounds(nz, tz, false);

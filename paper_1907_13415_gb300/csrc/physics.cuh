@@ -280,8 +280,8 @@ __host__ __device__ __forceinline__ void stress_tl(const T q[5], const T h[5], c
 // over gs/2, components 1, 2 and 4 over gs/4.  With N = 4/gs (xi D + W):
 // N_aa = 2 xi g_aa, N_ab = xi p + m, N_ba = xi p - m, p, m = g_ab +- g_ba; in
 // two dimensions every term with a z difference drops out (written out,
-// because the compiler may not drop products with zero).
-template <class T, int DIM>
+// because the compiler may not drop products with zero).  ADD: added to S.
+template <class T, int DIM, bool ADD = false>
 __host__ __device__ __forceinline__ void corotation_tl(const T q[5], const T g[3][3], T xi, T x2,
                                                        T S[5]) {
   constexpr bool D3 = DIM == 3;
@@ -301,20 +301,21 @@ __host__ __device__ __forceinline__ void corotation_tl(const T q[5], const T g[3
   }
   // 2 xi Q:G^T and -2 xi div u / 9 over gs/2
   const T tau = fma_(q[0], D3 ? n00 - n22 : n00, fma_(q[3], D3 ? n11 - n22 : n11, x2 * off));
-  const T tr = (D3 ? (n00 + n11) + n22 : n00 + n11) * T(-1.0 / 9.0);
+  const T div = D3 ? (n00 + n11) + n22 : n00 + n11;
+  auto add = [](T x, T y, const T& to) { return ADD ? fma_(x, y, to) : x * y; };
   const T a0 = n00 - tau, a1 = n11 - tau, a2 = D3 ? n22 - tau : -tau;
-  S[0] = fma_(a0, t00, fma_(N01, b, tr));
-  S[3] = fma_(a1, t11, fma_(N10, b, tr));
-  S[1] = fma_(a0 + a1, b, fma_(N01, t11, N10 * t00));
+  S[0] = fma_(a0, t00, fma_(N01, b, add(div, T(-1.0 / 9.0), S[0])));
+  S[3] = fma_(a1, t11, fma_(N10, b, add(div, T(-1.0 / 9.0), S[3])));
+  S[1] = fma_(a0 + a1, b, fma_(N01, t11, add(N10, t00, S[1])));
   if constexpr (D3) {
     S[0] = fma_(N02, c, S[0]);
     S[3] = fma_(N12, e, S[3]);
     S[1] = fma_(N02, e, fma_(N12, c, S[1]));
-    S[2] = fma_(a0 + a2, c, fma_(N01, e, fma_(N02, t22, fma_(N20, t00, N21 * b))));
-    S[4] = fma_(a1 + a2, e, fma_(N10, c, fma_(N12, t22, fma_(N20, b, N21 * t11))));
+    S[2] = fma_(a0 + a2, c, fma_(N01, e, fma_(N02, t22, fma_(N20, t00, add(N21, b, S[2])))));
+    S[4] = fma_(a1 + a2, e, fma_(N10, c, fma_(N12, t22, fma_(N20, b, add(N21, t11, S[4])))));
   } else {
-    S[2] = fma_(a0 + a2, c, N01 * e);
-    S[4] = fma_(a1 + a2, e, N10 * c);
+    S[2] = fma_(a0 + a2, c, add(N01, e, S[2]));
+    S[4] = fma_(a1 + a2, e, add(N10, c, S[4]));
   }
 }
 

@@ -15,14 +15,21 @@
 //     factors 1/2 and the stencils' weights go into constants formed once
 //     per lattice (CellPar), the collision works on sums and differences of
 //     opposite populations, Q Q and the gradient products use tracelessness;
+//     but the increments of Q are summed before they meet Q (two roundings
+//     at Q's size a step, after R(Q^n)/2 and after R(Q^P)/2), and the centre
+//     is taken out of the neighbour sums before they are scaled: otherwise
+//     every term rounds at Q's size, and the centre's rounded coefficient
+//     acts as a bias of Eq. 3 (against 80-bit arithmetic, 48^2 D2Q9, 60
+//     steps, paper parameters, median of 12 runs: largest error of Q 1.3e-16
+//     so, 2.5e-16 otherwise, at 1 to 2% of the step's time);
 //   - blocks of one warp over the linear cell index, so that small lattices
 //     reach as many SMs as they have warps and large ones leave no tail
 //     (two warps: 2-6% slower between 5,000 and 30,000 cells, else the same).
-// Float64 instructions per cell: D2Q9 114 + 79 + 71 + 120, D3Q19 175 + 156 +
-// 113 + 171.  Measured, tiled kernels -> these (us per step): 128 x 8 D2Q9
-// 55 -> 20, 256^2 D2Q9 114 -> 56 (48 at the issue rate above), 64^3 D3Q19
-// 830 -> 311 (300 at that rate; with float populations, whose conversions
-// run in integer arithmetic below, 312 instead of 329).
+// Float64 instructions per cell: D2Q9 119 + 79 + 72 + 121, D3Q19 180 + 156 +
+// 114 + 172.  Measured, tiled kernels -> these (us per step): 128 x 8 D2Q9
+// 55 -> 21, 256^2 D2Q9 114 -> 57 (48 at the issue rate above), 64^3 D3Q19
+// 830 -> 312 (308 at that rate; with float populations, whose conversions
+// run in integer arithmetic (convert.cuh), 312 instead of 329).
 #pragma once
 #include "common.cuh"
 #include "convert.cuh"
@@ -40,13 +47,14 @@ constexpr int CELL_T = 32;  // threads per block: one warp
 
 // Constants of one lattice.  The stencils give plain differences d~ and sums
 // s~ of neighbours (cell_stencil) with grad = gs/2 d~ and
-// lap = gs s~ - ls v; gs = 1, ls = 2 DIM for the standard stencils.
+// lap = gs (s~ - cs v); gs = 1, cs = 2 DIM for the standard stencils.
 struct CellPar {
   double rho0, inv_tau, keep;     // keep = 1 - 1/tau
-  double A1, Ag, Ag3, Kg;         // Eq. 3: A1 = -A0 (1 - gamma/3) - K ls, Kg = K gs
+  double A1, Ag, Ag3, Kg, cs;     // Eq. 3: Kg = K gs
   double s2, s23, sm, sp, sK;     // Eq. 5 times gs/2 (the stress is stored so scaled:
                                   // F = sum of its plain differences)
-  double xi, x2, Gamma, hs, qs, hu;  // Eq. 1: hs = gs/2, qs = gs/4, hu = -gs/2
+  double xi, x2, hs, qs, es;      // Eq. 1: hs = gs/2, qs = gs/4, es = gs/8
+  double Gh, Gq;                  // Gamma/hs, Gamma/qs
   double cC, cR, cB, cG;          // BGK: w2/tau, 3 w2/tau, 9 w2 k, 3 w2 k, k = 1 - 1/(2 tau)
 };
 
@@ -54,15 +62,15 @@ template <class Lat>
 inline CellPar make_cell_par(const Par<double>& p, bool iso) {
   constexpr double w2 = 1.0 / 36.0, w1 = Lat::DIM == 2 ? 1.0 / 9.0 : 1.0 / 18.0;
   const double gs = iso ? 6.0 * w1 : 1.0;
-  const double ls = iso ? 6.0 * (1.0 - Lat::w(0)) : 2.0 * Lat::DIM;
   CellPar c;
   c.rho0 = p.rho0;
   c.inv_tau = p.inv_tau;
   c.keep = 1.0 - p.inv_tau;
-  c.A1 = p.A1 - p.K * ls;
+  c.A1 = p.A1;
   c.Ag = p.Ag;
   c.Ag3 = p.Ag3;
   c.Kg = p.K * gs;
+  c.cs = iso ? (Lat::DIM == 2 ? 5.0 : 12.0) : 2.0 * Lat::DIM;  // sum of cell_stencil's weights
   const double f = 0.5 * gs;
   c.s2 = f * p.x2;
   c.s23 = f * p.x23;
@@ -71,10 +79,11 @@ inline CellPar make_cell_par(const Par<double>& p, bool iso) {
   c.sK = f * (p.K * gs * gs * 0.5);
   c.xi = p.xi;
   c.x2 = p.x2;
-  c.Gamma = p.Gamma;
   c.hs = 0.5 * gs;
   c.qs = 0.25 * gs;
-  c.hu = -0.5 * gs;
+  c.es = 0.125 * gs;
+  c.Gh = p.Gamma / c.hs;
+  c.Gq = p.Gamma / c.qs;
   c.cC = w2 * p.inv_tau;
   c.cR = 3.0 * w2 * p.inv_tau;
   c.cB = 9.0 * w2 * p.guo;
@@ -92,7 +101,7 @@ struct CellInst {
   double* q[2];   // padded Q, ping-pong
   double* u;      // padded u^n
   double* pi;     // stress times gs/2, dense [DIM DIM][n]
-  double* h;      // H(Q^n) for the predictor, then Q^n + Q^P for the corrector, dense [5][n]
+  double* h;      // H(Q^n) for the predictor, then Q^n + R(Q^n)/2 for the corrector, dense [5][n]
   double* qp;     // padded predictor Q^P
   const double* mrt;  // coefficients of collide_mrt_groups, or nullptr (BGK)
   unsigned block0;    // first block of this lattice in the launch
@@ -140,7 +149,10 @@ __device__ __forceinline__ void cell_stencil(const double* __restrict__ p, int64
 // H of Eq. 3 from q and the neighbour sums s
 __host__ __device__ __forceinline__ void cell_field(const double q[5], const double s[5],
                                                     const CellPar& c, double h[5]) {
-  molecular_field_tl(q, s, c.A1, c.Ag, c.Ag3, c.Kg, h);
+  double l[5];
+#pragma unroll
+  for (int k = 0; k < 5; k++) l[k] = fma(-c.cs, q[k], s[k]);
+  molecular_field_tl(q, l, c.A1, c.Ag, c.Ag3, c.Kg, h);
 }
 
 // Eq. 5 without P0, times gs/2, from the plain differences d[a][k]
@@ -151,23 +163,34 @@ __host__ __device__ __forceinline__ void cell_stress(const double q[5], const do
   stress_tl<double, DIM>(q, h, d, c.s2, c.s23, c.sm, c.sp, c.sK, P);
 }
 
-// r = base + R of Eq. 1 with its trace projected out, from q, h = H, u and the
-// plain differences d of Q and g[a][b] of u_a along b
-template <int DIM>
+// r = base + R (HALF: base + R/2) of Eq. 1 with its trace projected out, from
+// q, h = H, u and the plain differences d of Q and g[a][b] of u_a along b;
+// mid (if given) = base + R/2
+template <int DIM, bool HALF = false>
 __host__ __device__ __forceinline__ void cell_rhs(const double q[5], const double h[5],
                                                   const double d[3][5], const double u[3],
                                                   const double g[3][3], const CellPar& c,
-                                                  const double base[5], double r[5]) {
+                                                  const double base[5], double r[5],
+                                                  double* mid = nullptr) {
   constexpr bool D3 = DIM == 3;
+  // S starts as Gamma H - u.grad Q over the factor that scales S back, and
+  // the co-rotational term is added to it
   double S[5];
-  corotation_tl<double, DIM>(q, g, c.xi, c.x2, S);
-  const double u0 = c.hu * u[0], u1 = c.hu * u[1], u2 = D3 ? c.hu * u[2] : 0.0;
+  const double v0 = u[0] + u[0], v1 = u[1] + u[1], v2 = D3 ? u[2] + u[2] : 0.0;
 #pragma unroll
   for (int k = 0; k < 5; k++) {
-    double v = fma(c.Gamma, h[k], base[k]);
-    if constexpr (D3) v = fma(u2, d[2][k], v);
-    v = fma(u1, d[1][k], fma(u0, d[0][k], v));
-    r[k] = fma(k == 0 || k == 3 ? c.hs : c.qs, S[k], v);
+    const bool diag = k == 0 || k == 3;
+    double v = (diag ? c.Gh : c.Gq) * h[k];
+    if constexpr (D3) v = fma(diag ? -u[2] : -v2, d[2][k], v);
+    S[k] = fma(diag ? -u[1] : -v1, d[1][k], fma(diag ? -u[0] : -v0, d[0][k], v));
+  }
+  corotation_tl<double, DIM, true>(q, g, c.xi, c.x2, S);
+#pragma unroll
+  for (int k = 0; k < 5; k++) {
+    const bool diag = k == 0 || k == 3;
+    const double half = fma(diag ? c.qs : c.es, S[k], base[k]);
+    if (mid) mid[k] = half;
+    r[k] = HALF ? half : fma(diag ? c.hs : c.qs, S[k], base[k]);
   }
 }
 
@@ -309,7 +332,7 @@ __device__ __forceinline__ void cell_load(const double* __restrict__ p,
   }
 }
 
-// 3. predictor Q^P = Q^n + R(Q^n), and Q^n + Q^P for the corrector
+// 3. predictor Q^P = Q^n + R(Q^n), and Q^n + R(Q^n)/2 for the corrector
 template <class Lat, class G, bool ISO>
 __global__ void __launch_bounds__(CELL_T) k_cell_predict(const CellInst<G>* __restrict__ insts,
     int ninst, int cur) {
@@ -322,17 +345,17 @@ __global__ void __launch_bounds__(CELL_T) k_cell_predict(const CellInst<G>* __re
   const CellPar c = I->c;
   const Field<double> Q{I->q[cur], I->L};
   const int64_t o = Q.off(0, x, y, z), n = I->d.n;
-  double q[5], d[3][5], s[5], u[3], g[3][3], h[5], qp[5];
+  double q[5], d[3][5], s[5], u[3], g[3][3], h[5], qp[5], mid[5];
   cell_load<Lat, ISO>(Q.base + o, I->u + o, Q.L, q, d, s, u, g);
 #pragma unroll
   for (int k = 0; k < 5; k++) h[k] = I->h[k * n + idx];
-  cell_rhs<DIM>(q, h, d, u, g, c, q, qp);
+  cell_rhs<DIM>(q, h, d, u, g, c, q, qp, mid);
 #pragma unroll
-  for (int k = 0; k < 5; k++) I->h[k * n + idx] = q[k] + qp[k];
+  for (int k = 0; k < 5; k++) I->h[k * n + idx] = mid[k];
   store_with_images<double, 5, DIM>(Field<double>{I->qp, I->L}, I->d, x, y, z, qp);
 }
 
-// 4. corrector Q^{n+1} = [Q^n + Q^P + R(Q^P)]/2
+// 4. corrector Q^{n+1} = Q^n + [R(Q^n) + R(Q^P)]/2
 template <class Lat, class G, bool ISO>
 __global__ void __launch_bounds__(CELL_T) k_cell_correct(const CellInst<G>* __restrict__ insts,
     int ninst, int cur) {
@@ -350,9 +373,7 @@ __global__ void __launch_bounds__(CELL_T) k_cell_correct(const CellInst<G>* __re
 #pragma unroll
   for (int k = 0; k < 5; k++) base[k] = I->h[k * n + idx];
   cell_field(q, s, c, h);
-  cell_rhs<DIM>(q, h, d, u, g, c, base, r);
-#pragma unroll
-  for (int k = 0; k < 5; k++) r[k] *= 0.5;
+  cell_rhs<DIM, true>(q, h, d, u, g, c, base, r);
   store_with_images<double, 5, DIM>(Field<double>{I->q[cur ^ 1], I->L}, I->d, x, y, z, r);
 }
 

@@ -86,8 +86,10 @@ struct InstHost {
   Field<T> q[2];
   Field<T> u;
   int tz = 1;
-  T* mrt = nullptr;  // MRT coefficients s_k / |v_k|^2 on the device, or nullptr (BGK)
-  std::vector<double> mrt_coef;  // the same in float64
+  // MRT coefficients on the device, or nullptr (BGK): s_k / |v_k|^2 for the
+  // unfused schedule, then mrt_group_coef(s_k, k) for the step kernels
+  T* mrt = nullptr;
+  std::vector<double> rates;  // s_k
   // lazily allocated: unfused schedule, read-back staging, checkpoints
   T* pi = nullptr;
   Field<T> qp;
@@ -399,14 +401,17 @@ class Engine final : public EngineBase {
     cudaStream_t st = args_.stream;
     nlc_status s;
     if (rates) {
-      if (!I.mrt && (s = alloc(&I.mrt, (size_t)Q))) return s;
+      if (!I.mrt && (s = alloc(&I.mrt, (size_t)2 * Q))) return s;
       constexpr MomentBasis<Lat> B = make_moment_basis<Lat>();
-      T a[Q];
-      I.mrt_coef.resize(Q);
-      for (int k = 0; k < Q; k++) a[k] = (T)(I.mrt_coef[k] = rates[k] / B.n2[k]);
+      T a[2 * Q];
+      I.rates.assign(rates, rates + Q);
+      for (int k = 0; k < Q; k++) {
+        a[k] = (T)(rates[k] / B.n2[k]);
+        a[Q + k] = (T)mrt_group_coef<Lat, double>(rates[k], k);
+      }
       NLC_CK(cudaMemcpyAsync(I.mrt, a, sizeof(a), cudaMemcpyHostToDevice, st));
     }
-    const T* ptr = rates ? I.mrt : nullptr;
+    const T* ptr = rates ? I.mrt + Q : nullptr;
     NLC_CK(cudaMemcpyAsync(&insts_dev_[i].mrt, &ptr, sizeof(ptr), cudaMemcpyHostToDevice, st));
     NLC_CK(cudaStreamSynchronize(st));
     mrt_on_[i] = rates != nullptr;
@@ -1074,7 +1079,7 @@ class Engine final : public EngineBase {
         C.qp = I.qp.base;
         C.mrt = mrt_on_[i] ? cell_mrt_ + i * Q : nullptr;
         for (int k = 0; k < Q && mrt_on_[i]; k++)
-          rates[i * Q + k] = I.mrt_coef[k] * mrt_group_factor<Lat>(k);
+          rates[i * Q + k] = mrt_group_coef<Lat, double>(I.rates[k], k);
         C.block0 = (unsigned)nb;
         nb += (I.d.n + CELL_T - 1) / CELL_T;
       }

@@ -36,8 +36,8 @@ __host__ __device__ constexpr double mrt_group_factor(int k) {
   return 1.0;
 }
 
-// |v_k|^2 of the moment rows (make_moment_basis), as a switch that device
-// code can index at run time; 1 for the conserved rows, which are not used
+// |v_k|^2 of the moment rows (make_moment_basis); 1 for the conserved rows,
+// which are not used
 template <class Lat>
 __host__ __device__ constexpr double mrt_row_norm(int k) {
   if (Lat::DIM == 2) {
@@ -53,6 +53,39 @@ __host__ __device__ constexpr double mrt_row_norm(int k) {
   if (k == 12) return 8.0 / 3.0;
   if (k >= 13 && k <= 15) return 4.0;
   return k == 10 || k >= 16 ? 8.0 : 1.0;
+}
+
+// The coefficient of row k below is s_k over this whole number, |v_k|^2 over
+// mrt_group_factor, so that it is rounded once in either precision (rounding
+// s_k / |v_k|^2 and the factor first doubles its error in float32).
+template <class Lat>
+__host__ __device__ constexpr int mrt_group_norm(int k) {
+  if (Lat::DIM == 2) {
+    if (k == 1) return 12;
+    if (k == 2) return -12;
+    return k == 4 || k >= 6 ? 4 : 1;
+  }
+  if (k == 1) return 126;
+  if (k == 2) return -252;
+  if (k == 9) return 36;
+  if (k == 10) return 72;
+  if (k == 11) return 12;
+  if (k == 12) return 24;
+  if (k >= 13 && k <= 15) return 4;
+  return k == 4 || k == 6 || k == 8 || k >= 16 ? 8 : 1;
+}
+template <class Lat>
+constexpr bool mrt_norms_agree() {
+  for (int k = 0; k < Lat::Q; k++) {
+    const double d = mrt_group_norm<Lat>(k) * mrt_group_factor<Lat>(k) / mrt_row_norm<Lat>(k);
+    if (d < 1.0 - 1e-14 || d > 1.0 + 1e-14) return false;
+  }
+  return true;
+}
+static_assert(mrt_norms_agree<LatD2Q9>() && mrt_norms_agree<LatD3Q19>(), "mrt_group_norm");
+template <class Lat, class T>
+__host__ __device__ __forceinline__ T mrt_group_coef(T rate, int k) {
+  return rate / T(mrt_group_norm<Lat>(k));
 }
 
 // rho, drho = rho - rho0, J = sum c g and u = (J + F/2)/rho of Eq. 6 from the
@@ -138,8 +171,7 @@ __host__ __device__ __forceinline__ void collide_bgk_groups(T& g0, T* gi, T* gj,
 
 // g0, gi, gj: the rest population and the opposite pairs (pair_first and its
 // opposite), deviations, replaced by their post-collision values; drho = sum g,
-// J = sum c g, u = (J + F/2)/rho; a[k]: coefficients s_k / |v_k|^2 times
-// mrt_group_factor.  With y = g - g^eq + Ft/2 (Ft the source term),
+// J = sum c g, u = (J + F/2)/rho; a[k] = mrt_group_coef(s_k, k).  With y = g - g^eq + Ft/2 (Ft the source term),
 //   even part of y: -w (H0 + H_aa [+ H_bb +- H_ab]) beside g,
 //     H_aa = u_a t_a, H_ab = u_a t_b + u_b t_a, t = 9/2 (rho u - F),
 //     H0 = drho - sum H_aa / 3; its mass is zero, so y_0 = -(A + D);

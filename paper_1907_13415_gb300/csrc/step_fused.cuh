@@ -101,7 +101,7 @@ struct InstDev {
   G* g[2];         // populations (deviations), ping-pong
   Field<T> q[2];   // Q, ping-pong
   Field<T> u;      // u^n handed from the lb to the Beris-Edwards kernel
-  const T* mrt;    // Q coefficients s_k / |v_k|^2 of the MRT collision, or nullptr
+  const T* mrt;    // Q coefficients mrt_group_coef(s_k, k) of the MRT collision, or nullptr
 };
 
 // One thread block's work: a 32 x 8 (x, y) tile of instance `inst`, planes
@@ -347,8 +347,7 @@ __device__ __forceinline__ bool fused_lb_tile(const TileRef tile,
   __shared__ T s_mrt[MRT ? Lat::Q : 1];
   if constexpr (MRT) {
     if (tid < Lat::Q)
-      s_mrt[tid] = (I.mrt ? I.mrt[tid] : I.p.inv_tau / T(mrt_row_norm<Lat>(tid))) *
-                   T(mrt_group_factor<Lat>(tid));
+      s_mrt[tid] = I.mrt ? I.mrt[tid] : mrt_group_coef<Lat, T>(I.p.inv_tau, tid);
   }
   if (tid == 0) {
     for (int s = 0; s < C::NSQ; s++) mbar_init(&bars[s], 1);

@@ -30,6 +30,14 @@ static void field(const double* p, bool iso, const double* q, const double* s, d
 }
 
 extern "C" {
+// coefficient of the grouped MRT collision, and |v_k|^2 over the row's factor
+float hr_mrt_coef(int d3, float rate, int k) {
+  return d3 ? mrt_group_coef<LatD3Q19, float>(rate, k) : mrt_group_coef<LatD2Q9, float>(rate, k);
+}
+double hr_mrt_norm(int d3, int k) {
+  return d3 ? mrt_row_norm<LatD3Q19>(k) / mrt_group_factor<LatD3Q19>(k)
+            : mrt_row_norm<LatD2Q9>(k) / mrt_group_factor<LatD2Q9>(k);
+}
 // Eq. 1 from the plain differences d[3][5], g[3][3] (standard stencils)
 void hr_rhs(int d3, const double* p, const double* q, const double* h, const double* d,
             const double* u, const double* g, const double* base, double* r) {

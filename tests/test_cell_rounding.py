@@ -1,6 +1,7 @@
-"""Rounding of the float64 cell formulas (csrc/step_cell.cuh), compiled for
-the host, against extended precision: Q meets its increment in one rounding,
-and a uniform field has no Laplacian."""
+"""Rounding of pointwise formulas, compiled for the host: in the float64 cell
+kernels (csrc/step_cell.cuh) Q meets its increment in one rounding and a
+uniform field has no Laplacian; the coefficients of the grouped MRT collision
+(csrc/mrt.cuh) are rounded once."""
 import ctypes
 import os
 import shutil
@@ -90,3 +91,18 @@ def test_a_uniform_field_has_no_laplacian(hr, d3, iso):
             p = np.array([0.1, K, 2.7, 0.34, 0.8, 1.5])
             hr.hr_field(d3, iso, P(p), P(q), P(s), P(h[k]))
         assert np.array_equal(h[0], h[1])
+
+
+@pytest.mark.parametrize("d3", [0, 1], ids=["d2q9", "d3q19"])
+def test_mrt_coefficients_are_rounded_once(hr, d3):
+    hr.hr_mrt_coef.restype, hr.hr_mrt_coef.argtypes = ctypes.c_float, [ctypes.c_int, ctypes.c_float,
+                                                                       ctypes.c_int]
+    hr.hr_mrt_norm.restype = ctypes.c_double
+    conserved = (0, 3, 5, 7) if d3 else (0, 3, 5)
+    rng = np.random.default_rng(13)
+    for rate in rng.uniform(0.05, 1.95, 200).astype(np.float32):
+        for k in range(19 if d3 else 9):
+            if k not in conserved:
+                exact = float(rate) / hr.hr_mrt_norm(d3, k)
+                got = np.float32(hr.hr_mrt_coef(d3, rate, k))
+                assert abs(float(got) - exact) <= 0.5000001 * float(np.spacing(np.abs(got)))

@@ -110,13 +110,7 @@ __host__ __device__ __forceinline__ void moments_groups(T g0, const T* gi, const
     }
   }
   rho = rho0 + drho;
-  T inv;
-#ifdef __CUDA_ARCH__
-  if constexpr (sizeof(T) == 4)
-    inv = __fdividef(1.0f, rho);  // hardware reciprocal, 2 ulp, no slow path
-  else
-#endif
-    inv = T(1) / rho;
+  const T inv = T(1) / rho;
 #pragma unroll
   for (int a = 0; a < Lat::DIM; a++) u[a] = fma_(T(0.5), F[a], J[a]) * inv;
 }

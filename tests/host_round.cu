@@ -1,5 +1,5 @@
-// Host build of pointwise formulas, for CPU tests of their rounding.  Test
-// infrastructure only.
+// Host (and, for the density's reciprocal, device) build of pointwise
+// formulas, for tests of their rounding.  Test infrastructure only.
 #include "../paper_1907_13415_gb300/csrc/step_cell.cuh"
 
 using namespace nlc;
@@ -29,7 +29,27 @@ static void field(const double* p, bool iso, const double* q, const double* s, d
   cell_field(q, s, make_cell_par<Lat>(par(p), iso), h);
 }
 
+// rho and u_x = J_x / rho of n cells with J_x = 1, by moments_groups
+template <class Lat>
+__global__ void k_velocity(int n, const float* rho0, float* rho, float* ux) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  constexpr int NP = (Lat::Q - 1) / 2;
+  float gi[NP] = {1.0f}, gj[NP] = {}, F[3] = {}, drho, J[3], u[3];
+  moments_groups<Lat, float>(0.0f, gi, gj, F, rho0[i], rho[i], drho, J, u);
+  ux[i] = u[0];
+}
+
 extern "C" {
+// device arrays of n floats
+int hr_velocity(int d3, int n, const float* rho0, float* rho, float* ux) {
+  const int blocks = (n + 127) / 128;
+  if (d3)
+    k_velocity<LatD3Q19><<<blocks, 128>>>(n, rho0, rho, ux);
+  else
+    k_velocity<LatD2Q9><<<blocks, 128>>>(n, rho0, rho, ux);
+  return (int)cudaDeviceSynchronize();
+}
 // coefficient of the grouped MRT collision, and |v_k|^2 over the row's factor
 float hr_mrt_coef(int d3, float rate, int k) {
   return d3 ? mrt_group_coef<LatD3Q19, float>(rate, k) : mrt_group_coef<LatD2Q9, float>(rate, k);

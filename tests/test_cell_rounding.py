@@ -1,7 +1,8 @@
 """Rounding of pointwise formulas, compiled for the host: in the float64 cell
 kernels (csrc/step_cell.cuh) Q meets its increment in one rounding and a
 uniform field has no Laplacian; the coefficients of the grouped MRT collision
-(csrc/mrt.cuh) are rounded once."""
+(csrc/mrt.cuh) are rounded once, and its velocity is divided by the density
+without an approximate reciprocal."""
 import ctypes
 import os
 import shutil
@@ -21,7 +22,7 @@ def hr(tmp_path_factory):
     if not os.path.exists(nvcc):
         pytest.skip("nvcc not available")
     out = tmp_path_factory.mktemp("hr") / "libhr.so"
-    subprocess.check_call([nvcc, "-O1", "-std=c++17", "--expt-relaxed-constexpr",
+    subprocess.check_call([nvcc, "-O1", "-std=c++17", "--expt-relaxed-constexpr", "-ftz=true",
                            "-gencode", "arch=compute_103a,code=sm_103a", "-Xcompiler", "-fPIC",
                            "-I", os.path.join(os.path.dirname(HERE), "include"),
                            "-shared", os.path.join(HERE, "host_round.cu"), "-o", str(out)])
@@ -106,3 +107,20 @@ def test_mrt_coefficients_are_rounded_once(hr, d3):
                 exact = float(rate) / hr.hr_mrt_norm(d3, k)
                 got = np.float32(hr.hr_mrt_coef(d3, rate, k))
                 assert abs(float(got) - exact) <= 0.5000001 * float(np.spacing(np.abs(got)))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d3", [0, 1], ids=["d2q9", "d3q19"])
+def test_velocity_is_divided_by_the_density_exactly(hr, d3):
+    """J = 1, so u is 1/rho, correctly rounded."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    rng = np.random.default_rng(14)
+    rho0 = torch.from_numpy(rng.uniform(-0.3, 0.7, 100000).astype(np.float32)).cuda()
+    rho, ux = torch.empty_like(rho0), torch.empty_like(rho0)
+    torch.cuda.synchronize()
+    assert hr.hr_velocity(d3, rho0.numel(), *(ctypes.c_void_p(t.data_ptr())
+                                              for t in (rho0, rho, ux))) == 0
+    rho, ux = rho.cpu().numpy(), ux.cpu().numpy()
+    assert np.array_equal(ux, np.float32(1) / rho)

@@ -337,7 +337,9 @@ NLC_API nlc_status nlc_get_populations(nlc_ctx* ctx, int32_t inst, double* f);
  * may be scheduled while the kernel before it in the stream (the caller's
  * own, too) is finishing, and waits on the device for that kernel to
  * complete before it touches memory that kernels write, so stream order
- * holds for every buffer. */
+ * holds for every buffer.  Steps in a caller's stream capture keep the
+ * stencils and the choice between BGK and MRT kernels of the capture;
+ * parameters and rates are read from device memory at every replay. */
 NLC_API nlc_status nlc_step(nlc_ctx* ctx, int64_t n);
 
 /* Computes the observables of the current state of instance inst into *out

@@ -437,12 +437,9 @@ class Engine final : public EngineBase {
 
   // stencils of every lattice: standard (false) or isotropic (true)
   nlc_status set_stencil(bool iso) override {
-    if (iso != iso_) {
-      drop_graphs();
-      cells_stale_ = true;
-    }
+    if (iso != iso_) drop_graphs();
     iso_ = iso;
-    return cells_dev_ ? ensure_cells() : NLC_OK;
+    return NLC_OK;
   }
 
   nlc_status set_params(int i, const nlc_params& q) override {
@@ -453,12 +450,13 @@ class Engine final : public EngineBase {
     NLC_CK(cudaMemcpyAsync(&insts_dev_[i].p, &I.p, sizeof(Par<T>), cudaMemcpyHostToDevice,
                            args_.stream));
     if constexpr (kCell) {
-      if (cells_dev_ && !cells_stale_) {
-        const CellPar c = make_cell_par<Lat>(I.p, iso_);
-        NLC_CK(cudaMemcpyAsync(&cells_dev_[i].c, &c, sizeof(c), cudaMemcpyHostToDevice,
-                               args_.stream));
-        NLC_CK(cudaStreamSynchronize(args_.stream));
-      }
+      if (cells_dev_ && !cells_stale_)
+        for (int k = 0; k < 2; k++) {
+          const CellPar c = make_cell_par<Lat>(I.p, k != 0);
+          NLC_CK(cudaMemcpyAsync(&cells_dev_[k * inst_.size() + i].c, &c, sizeof(c),
+                                 cudaMemcpyHostToDevice, args_.stream));
+          NLC_CK(cudaStreamSynchronize(args_.stream));
+        }
     }
     NLC_CK(cudaStreamSynchronize(args_.stream));
     return NLC_OK;
@@ -1058,9 +1056,9 @@ class Engine final : public EngineBase {
         }
         if (s) return s;
       }
-      if (!cells_dev_ && (s = alloc(&cells_dev_, n))) return s;
+      if (!cells_dev_ && (s = alloc(&cells_dev_, 2 * n))) return s;
       if (any_mrt_ && !cell_mrt_ && (s = alloc(&cell_mrt_, n * Q))) return s;
-      std::vector<CellInst<G>> ci(n);
+      std::vector<CellInst<G>> ci(2 * n);
       std::vector<double> rates(n * Q, 0.0);
       int64_t nb = 0;
       for (size_t i = 0; i < n; i++) {
@@ -1068,7 +1066,7 @@ class Engine final : public EngineBase {
         CellInst<G>& C = ci[i];
         C.d = I.d;
         C.L = I.L;
-        C.c = make_cell_par<Lat>(I.p, iso_);
+        C.c = make_cell_par<Lat>(I.p, false);
         for (int b = 0; b < 2; b++) {
           C.g[b] = I.g[b];
           C.q[b] = I.q[b].base;
@@ -1082,6 +1080,8 @@ class Engine final : public EngineBase {
           rates[i * Q + k] = mrt_group_coef<Lat, double>(I.rates[k], k);
         C.block0 = (unsigned)nb;
         nb += (I.d.n + CELL_T - 1) / CELL_T;
+        ci[n + i] = C;
+        ci[n + i].c = make_cell_par<Lat>(I.p, true);
       }
       if (nb > INT32_MAX) {
         cells_off_ = true;
@@ -1092,7 +1092,7 @@ class Engine final : public EngineBase {
       if (any_mrt_)
         NLC_CK(cudaMemcpyAsync(cell_mrt_, rates.data(), sizeof(double) * n * Q,
                                cudaMemcpyHostToDevice, st));
-      NLC_CK(cudaMemcpyAsync(cells_dev_, ci.data(), sizeof(CellInst<G>) * n,
+      NLC_CK(cudaMemcpyAsync(cells_dev_, ci.data(), sizeof(CellInst<G>) * 2 * n,
                              cudaMemcpyHostToDevice, st));
       NLC_CK(cudaStreamSynchronize(st));
       cells_stale_ = false;
@@ -1106,10 +1106,10 @@ class Engine final : public EngineBase {
       int e[5];
       auto at = [&](int k) { e[k] = mark(); };
       const cudaError_t r =
-          iso_ ? launch_cell_step<Lat, G, true>(cells_dev_, (int)inst_.size(), cell_blocks_, cur_,
-                                                st, at)
-               : launch_cell_step<Lat, G, false>(cells_dev_, (int)inst_.size(), cell_blocks_, cur_,
-                                                 st, at);
+          iso_ ? launch_cell_step<Lat, G, true>(cells_dev_ + inst_.size(), (int)inst_.size(),
+                                                cell_blocks_, cur_, any_mrt_, st, at)
+               : launch_cell_step<Lat, G, false>(cells_dev_, (int)inst_.size(), cell_blocks_,
+                                                 cur_, any_mrt_, st, at);
       if (r != cudaSuccess) {
         err = std::string("cell kernels: ") + cudaGetErrorString(r);
         return NLC_ECUDA;
@@ -1544,7 +1544,8 @@ class Engine final : public EngineBase {
   double* hwords_ = nullptr;  // host_words
   size_t hwords_n_ = 0;
   bool hwords_locked_ = false;
-  // float64 arithmetic: descriptors of the cell kernels (ensure_cells)
+  // float64 arithmetic: descriptors of the cell kernels (ensure_cells), of
+  // every lattice with the standard, then with the isotropic stencils
   CellInst<G>* cells_dev_ = nullptr;
   double* cell_mrt_ = nullptr;   // [lattices][Q]
   unsigned cell_blocks_ = 0;

@@ -242,10 +242,11 @@ __global__ void __launch_bounds__(CELL_T) k_cell_stress(const CellInst<G>* __res
     for (int b = 0; b < DIM; b++) I->pi[(a * DIM + b) * n + idx] = P[a][b];
 }
 
-// 2. F, the pulled populations, rho and u, the collision
+// 2. F, the pulled populations, rho and u, the collision (BGK on every lattice
+// unless mrt)
 template <class Lat, class G, bool ISO>
 __global__ void __launch_bounds__(CELL_T) k_cell_lb(const CellInst<G>* __restrict__ insts,
-    int ninst, int cur) {
+    int ninst, int cur, int mrt) {
   constexpr int DIM = Lat::DIM, NP = (Lat::Q - 1) / 2;
   grid_dep_wait();
   const CellInst<G>* I;
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(CELL_T) k_cell_lb(const CellInst<G>* __restric
   double rho, drho, J[3], u[3];
   moments_groups<Lat, double>(g0, gi, gj, F, c.rho0, rho, drho, J, u);
   auto put = [&](int i, double v) { gout[i * d.n + idx] = store_as<G>(v); };
-  if (I->mrt)
+  if (mrt && I->mrt)
     collide_mrt_groups<Lat, double>(g0, gi, gj, rho, drho, J, u, F, I->mrt);
   else
     collide_bgk_groups<Lat, double>(g0, gi, gj, rho, drho, u, F, c.keep, c.cC, c.cR, c.cB, c.cG);
@@ -383,18 +384,21 @@ __global__ void __launch_bounds__(CELL_T) k_cell_correct(const CellInst<G>* __re
 // one runs go wherever an SM has room, and the uneven spread costs more than
 // the launch gap (256^2 D2Q9: 90 us per step with the trigger, 56 without,
 // 57 with plain launches).
+// mrt: some lattice of the launch takes the MRT collision.  The stencils and
+// this choice are arguments of the launch, so that steps in a caller's stream
+// capture keep those of the capture, whatever is set later.
 // mark(k) is called before kernel k and mark(4) after the last.
 template <class Lat, class G, bool ISO, class Mark>
 cudaError_t launch_cell_step(const CellInst<G>* insts, int ninst, unsigned nblocks, int cur,
-                             cudaStream_t st, Mark mark) {
+                             bool mrt, cudaStream_t st, Mark mark) {
   int k = 0;
-  auto run = [&](auto kernel) {
+  auto run = [&](auto kernel, auto... more) {
     mark(k++);
-    return launch_pdl(kernel, (int)nblocks, CELL_T, 0, st, insts, ninst, cur);
+    return launch_pdl(kernel, (int)nblocks, CELL_T, 0, st, insts, ninst, cur, more...);
   };
   cudaError_t e;
   if ((e = run(k_cell_stress<Lat, G, ISO>)) != cudaSuccess) return e;
-  if ((e = run(k_cell_lb<Lat, G, ISO>)) != cudaSuccess) return e;
+  if ((e = run(k_cell_lb<Lat, G, ISO>, mrt ? 1 : 0)) != cudaSuccess) return e;
   if ((e = run(k_cell_predict<Lat, G, ISO>)) != cudaSuccess) return e;
   if ((e = run(k_cell_correct<Lat, G, ISO>)) != cudaSuccess) return e;
   mark(4);

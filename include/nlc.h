@@ -245,9 +245,9 @@ NLC_API nlc_status nlc_set_check(nlc_ctx* ctx, int32_t every);
  * launched it fails with NLC_ETIMEOUT; the fault is cleared once reported
  * and the context stays usable (its state is that of the last completed
  * call, except for the adjoint's own work arrays).  ns < 0 restores the
- * default, 200 ms; 0 makes any wait that does not find the barrier already
- * complete run out (a test of the path).  Waits on tile copies inside the
- * step kernels keep their own fixed 200 ms bound. */
+ * default, 200 ms; 0 makes the wait of every block run out that does not
+ * arrive at the barrier as the last one (a test of the path).  Waits on tile
+ * copies inside the step kernels keep their own fixed 200 ms bound. */
 NLC_API nlc_status nlc_set_wait_budget(nlc_ctx* ctx, int64_t ns);
 
 /* Selects the kernel schedule (NLC_SCHED_*) for later nlc_step calls. */

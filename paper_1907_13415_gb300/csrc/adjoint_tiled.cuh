@@ -249,14 +249,14 @@ __global__ void __maxnreg__(96) k_seg_reverse_tiled(SegArgs<T> a, int tiles_x) {
     }
     // the adjoints of step j's state are complete everywhere before the
     // next reverse step reads them around every tile
-    grid_arrive(a.bar);
+    const bool may_wait = grid_arrive(a.bar, gen, a.wait_ns);
     if (own) {
       const T terms[9] = {S.qp[0][t], S.qp[1][t], S.qp[2][t], S.qp[3][t], S.qp[4][t],
                           S.ua[0][t], S.ua[1][t], S.gv[0][t], S.gv[1][t]};
 #pragma unroll
       for (int k = 0; k < 9; k++) acc3[k % 3] += widen(terms[k]);
     }
-    if (!(ok = grid_wait(a.bar, gen, a.err, a.wait_ns))) break;
+    if (!(ok = grid_wait(a.bar, gen, a.err, a.wait_ns, may_wait))) break;
     lc ^= 1;
   }
   if (!ok) return;

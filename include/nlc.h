@@ -149,7 +149,10 @@ typedef struct nlc_ctx nlc_ctx;
  * The fused kernels address the populations with 32-bit offsets when every
  * lattice of the context has q nx ny nz < 2^32, else with 64-bit ones; the
  * environment variable NLC_POP_INDEX64=1, read here, forces the 64-bit form
- * (both give the same step bit for bit).
+ * (both give the same step bit for bit).  The environment variable
+ * NLC_ALLOC_LIMIT, read here, caps the bytes of device memory that the context
+ * holds: a call that needs more fails with NLC_ENOMEM and leaves the state as
+ * it was.
  * Errors: NLC_EINVAL (bad sizes or parameters, D2Q9 with nz != 1),
  * NLC_ENOMEM, NLC_ECUDA. */
 NLC_API nlc_status nlc_create(const nlc_grid* grid, const nlc_params* params,

@@ -140,7 +140,12 @@ class Engine final : public EngineBase {
   // float64 arithmetic: the fused schedule runs the kernels of step_cell.cuh
   static constexpr bool kCell = std::is_same<T, double>::value;
 
-  explicit Engine(const EngineArgs& a) : args_(a) {}
+  explicit Engine(const EngineArgs& a) : args_(a) {
+    if (const char* w = std::getenv("NLC_ALLOC_LIMIT")) {
+      const unsigned long long b = std::strtoull(w, nullptr, 10);
+      if (b > 0) limit_ = (size_t)b;
+    }
+  }
 
   ~Engine() override {
     for (int c = 0; c < 2; c++)
@@ -150,7 +155,7 @@ class Engine final : public EngineBase {
     if (side_stream_) cudaStreamDestroy(side_stream_);
     for (cudaEvent_t e : seg_ev_)
       if (e) cudaEventDestroy(e);
-    for (void* ptr : allocs_) cudaFree(ptr);
+    for (const Block& b : allocs_) cudaFree(b.ptr);
     free_host_words();
   }
 
@@ -218,11 +223,12 @@ class Engine final : public EngineBase {
   nlc_status set_chunk(int tz, bool taper) override {
     cudaStream_t st = args_.stream;
     std::vector<TileRef> tiles;
-    taper_ = taper;
+    std::vector<int> depth(inst_.size());
     for (size_t i = 0; i < inst_.size(); i++) {
-      InstHost<T, G>& I = inst_[i];
-      I.tz = tz > 0 ? std::min(tz, column_length<Lat>(I.d))
-                    : fused_tz<Lat>(I.d, (int64_t)tiles.size());
+      const InstHost<T, G>& I = inst_[i];
+      int& z = depth[i];
+      z = tz > 0 ? std::min(tz, column_length<Lat>(I.d))
+                 : fused_tz<Lat>(I.d, (int64_t)tiles.size());
       if (tz <= 0 && DIM == 3 && !kCell && inst_.size() == 1) {
         // the estimate covers one float32 D3Q19 lattice with the device to
         // itself (us per step at its depth / the rule above: 128^3 177 / 199,
@@ -231,22 +237,22 @@ class Engine final : public EngineBase {
         NLC_CK(cudaGetDevice(&dev));
         NLC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         const long columns = (long)((I.d.nx + FTX - 1) / FTX) * ((I.d.ny + FTY - 1) / FTY);
-        I.tz = estimated_depth(I.d.nz, columns, sms, I.tz);
+        z = estimated_depth(I.d.nz, columns, sms, z);
       }
-      append_tiles<Lat>((int)i, I.d, I.tz, taper_, &tiles);
+      append_tiles<Lat>((int)i, I.d, z, taper, &tiles);
     }
     NLC_CK(cudaStreamSynchronize(st));  // no step may still read the old list
     if (tiles.size() > tiles_cap_) {
-      if (tiles_dev_) {
-        cudaFree(tiles_dev_);
-        allocs_.erase(std::remove(allocs_.begin(), allocs_.end(), (void*)tiles_dev_),
-                      allocs_.end());
-        tiles_dev_ = nullptr;
-      }
-      nlc_status s = alloc(&tiles_dev_, tiles.size());
+      // the old list stays until there is a new one
+      TileRef* list = nullptr;
+      nlc_status s = alloc(&list, tiles.size());
       if (s) return s;
+      release(tiles_dev_);
+      tiles_dev_ = list;
       tiles_cap_ = tiles.size();
     }
+    taper_ = taper;
+    for (size_t i = 0; i < inst_.size(); i++) inst_[i].tz = depth[i];
     ntiles_ = (int)tiles.size();
     NLC_CK(cudaMemcpyAsync(tiles_dev_, tiles.data(), sizeof(TileRef) * tiles.size(),
                            cudaMemcpyHostToDevice, st));
@@ -718,9 +724,11 @@ class Engine final : public EngineBase {
   nlc_status load_state(const void* src) override {
     cudaStream_t st = args_.stream;
     const char* in = (const char*)src;
-    for (auto& I : inst_) {
+    for (auto& I : inst_) {  // before any lattice is changed
       nlc_status s;
       if (!I.raw && (s = alloc(&I.raw, (size_t)5 * I.d.n))) return s;
+    }
+    for (auto& I : inst_) {
       const int64_t n = I.d.n;
       NLC_CK(cudaMemcpyAsync(I.g[0], in, sizeof(G) * Q * n, cudaMemcpyHostToDevice, st));
       in += sizeof(G) * Q * n;
@@ -749,7 +757,7 @@ class Engine final : public EngineBase {
     cudaStream_t st = args_.stream;
     nlc_status s;
     if ((s = ensure_staging(I)) || (s = ensure_segment(I, ckpt_every)) ||
-        (s = ensure_adjoint(I, nseg + 1)))
+        (s = ensure_adjoint(I, nseg + 1)) || (s = obs_fused() ? ensure_obs_tiles(0) : NLC_OK))
       return s;
     if (I.seg_grid <= 0) {
       err = "the adjoint needs cooperative launches of its segment kernels";
@@ -846,35 +854,11 @@ class Engine final : public EngineBase {
     const double s_ref = 1.0 / 3.0;
     const double* partial = nullptr;
     int nblocks = 0;
-    if (!kCell && maps_ok_ && !iso_ && ix32_) {
+    if (obs_fused()) {
       if constexpr (!kCell) {
       // one pass of the fused lb kernel in its observing form over this
       // lattice's tiles (the step's tile machinery, nothing stored)
-      // the lattice's tiles in the chunk list the step runs with (the
-      // autotuner's choice when it ran)
-      if (!I.obs_tiles || I.obs_tz != I.tz || I.obs_taper != taper_) {
-        std::vector<TileRef> tl;
-        append_tiles<Lat>(i, I.d, I.tz, taper_, &tl);
-        if (tl.size() > I.obs_cap) {
-          for (void* old : {(void*)I.obs_tiles, (void*)I.obs_part})
-            if (old) {
-              NLC_CK(cudaStreamSynchronize(st));
-              cudaFree(old);
-              allocs_.erase(std::remove(allocs_.begin(), allocs_.end(), old), allocs_.end());
-            }
-          I.obs_tiles = nullptr;
-          I.obs_part = nullptr;
-          if ((s = alloc(&I.obs_tiles, tl.size())) ||
-              (s = alloc(&I.obs_part, (tl.size() + 1) * OBS_SLOTS)))
-            return s;
-          I.obs_cap = tl.size();
-        }
-        NLC_CK(cudaMemcpyAsync(I.obs_tiles, tl.data(), sizeof(TileRef) * tl.size(),
-                               cudaMemcpyHostToDevice, st));
-        I.obs_ntiles = (int)tl.size();
-        I.obs_tz = I.tz;
-        I.obs_taper = taper_;
-      }
+      if ((s = ensure_obs_tiles(i))) return s;
       cudaError_t e = launch_fused_obs<Lat, T>(insts_dev_, qmaps_dev_, I.obs_tiles, I.obs_ntiles,
                                                cur_, derr_, I.obs_part, st);
       if (e != cudaSuccess) {
@@ -932,18 +916,55 @@ class Engine final : public EngineBase {
 
   template <class U>
   nlc_status alloc(U** p, size_t count) {
+    const size_t bytes = sizeof(U) * (count ? count : 1);
+    if (bytes > limit_ - held_) {
+      err = "device memory limit of the context: needs " + std::to_string(held_ + bytes) + " bytes";
+      return NLC_ENOMEM;
+    }
     void* ptr = nullptr;
-    cudaError_t e = cudaMalloc(&ptr, sizeof(U) * (count ? count : 1));
+    cudaError_t e = cudaMalloc(&ptr, bytes);
     if (e != cudaSuccess) {
-      err = std::string("cudaMalloc(") + std::to_string(sizeof(U) * count) +
+      err = std::string("cudaMalloc(") + std::to_string(bytes) +
             " bytes): " + cudaGetErrorString(e);
       cudaGetLastError();
       return e == cudaErrorMemoryAllocation ? NLC_ENOMEM : NLC_ECUDA;
     }
-    allocs_.push_back(ptr);
+    allocs_.push_back({ptr, bytes});
+    held_ += bytes;
     *p = (U*)ptr;
     return NLC_OK;
   }
+
+  // gives one allocation back (nothing for nullptr)
+  void release(void* p) {
+    for (size_t k = 0; p && k < allocs_.size(); k++)
+      if (allocs_[k].ptr == p) {
+        cudaFree(p);
+        held_ -= allocs_[k].bytes;
+        allocs_.erase(allocs_.begin() + k);
+        return;
+      }
+  }
+
+  // Allocations that belong together: given back unless all of them are kept.
+  // A pointer of the engine is set only once its whole group is there, so that
+  // a call which fails for lack of memory leaves nothing half made behind.
+  struct Group {
+    Engine& e;
+    std::vector<void*> own;
+    bool kept = false;
+    explicit Group(Engine& eng) : e(eng) {}
+    ~Group() {
+      if (!kept)
+        for (void* p : own) e.release(p);
+    }
+    template <class U>
+    nlc_status alloc(U** p, size_t count) {
+      const nlc_status s = e.alloc(p, count);
+      if (!s) own.push_back(*p);
+      return s;
+    }
+  };
 
   // page-locked host words for small results (one copy, no staging by the
   // driver); plain memory where none can be locked.  Kept by the engine and
@@ -1007,23 +1028,15 @@ class Engine final : public EngineBase {
     nlc_status s;
     const int64_t n = I.d.n;
     T *pi = nullptr, *qp = nullptr, *r1 = nullptr;
-    if ((s = alloc(&pi, (size_t)DIM * DIM * n)) || (s = alloc(&qp, (size_t)5 * I.L.comp)) ||
-        (s = alloc(&r1, (size_t)5 * n))) {
-      release(pi);
-      release(qp);
+    Group mem(*this);
+    if ((s = mem.alloc(&pi, (size_t)DIM * DIM * n)) || (s = mem.alloc(&qp, (size_t)5 * I.L.comp)) ||
+        (s = mem.alloc(&r1, (size_t)5 * n)))
       return s;
-    }
+    mem.kept = true;
     I.pi = pi;
     I.qp = Field<T>{qp, I.L};
     I.r1 = r1;
     return NLC_OK;
-  }
-
-  // gives one allocation back (nothing for nullptr)
-  void release(void* p) {
-    if (!p) return;
-    cudaFree(p);
-    allocs_.erase(std::remove(allocs_.begin(), allocs_.end(), p), allocs_.end());
   }
 
   // float64 arithmetic: the workspaces (those of the unfused schedule) and
@@ -1127,20 +1140,63 @@ class Engine final : public EngineBase {
     if (I.stage) return NLC_OK;
     nlc_status s;
     const int64_t n = I.d.n;
-    if ((s = alloc(&I.stage, (size_t)9 * n))) return s;
     if ((s = ensure_unfused(I))) return s;
     int dev = 0, sms = 0;
     NLC_CK(cudaGetDevice(&dev));
     NLC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t want = (n + 255) / 256;
-    I.obs_blocks = (int)(want < 16 * sms ? want : 16 * sms);
-    if (I.obs_blocks < 1) I.obs_blocks = 1;
-    if ((s = alloc(&I.partial, (size_t)(I.obs_blocks + 1) * OBS_SLOTS))) return s;
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(want, 16 * sms));
     const int64_t rows = (int64_t)I.d.ny * I.d.nz;
     const int rpc = profile_rows_per_chunk(I.d);
     const int64_t nchunks = (rows + rpc - 1) / rpc;
-    if ((s = alloc(&I.prof_partial, (size_t)(nchunks * I.d.nx)))) return s;
-    if ((s = alloc(&I.res, OBS_SLOTS + (size_t)I.d.nx + 1))) return s;
+    double *stage = nullptr, *partial = nullptr, *prof = nullptr, *res = nullptr;
+    Group mem(*this);
+    if ((s = mem.alloc(&stage, (size_t)9 * n)) ||
+        (s = mem.alloc(&partial, (size_t)(blocks + 1) * OBS_SLOTS)) ||
+        (s = mem.alloc(&prof, (size_t)(nchunks * I.d.nx))) ||
+        (s = mem.alloc(&res, OBS_SLOTS + (size_t)I.d.nx + 1)))
+      return s;
+    mem.kept = true;
+    I.stage = stage;
+    I.obs_blocks = blocks;
+    I.partial = partial;
+    I.prof_partial = prof;
+    I.res = res;
+    return NLC_OK;
+  }
+
+  // observables by the fused lb kernel rather than one cell per thread
+  bool obs_fused() const { return !kCell && maps_ok_ && !iso_ && ix32_; }
+
+  // tiles of lattice i alone for the observing form of the fused lb kernel, in
+  // the chunk list the step runs with (the autotuner's choice when it ran)
+  nlc_status ensure_obs_tiles(int i) {
+    InstHost<T, G>& I = inst_[i];
+    if (I.obs_tiles && I.obs_tz == I.tz && I.obs_taper == taper_) return NLC_OK;
+    cudaStream_t st = args_.stream;
+    nlc_status s;
+    std::vector<TileRef> tl;
+    append_tiles<Lat>(i, I.d, I.tz, taper_, &tl);
+    if (tl.size() > I.obs_cap) {
+      TileRef* list = nullptr;
+      double* part = nullptr;
+      Group mem(*this);
+      if ((s = mem.alloc(&list, tl.size())) ||
+          (s = mem.alloc(&part, (tl.size() + 1) * OBS_SLOTS)))
+        return s;
+      mem.kept = true;
+      NLC_CK(cudaStreamSynchronize(st));
+      release(I.obs_tiles);
+      release(I.obs_part);
+      I.obs_tiles = list;
+      I.obs_part = part;
+      I.obs_cap = tl.size();
+    }
+    NLC_CK(cudaMemcpyAsync(I.obs_tiles, tl.data(), sizeof(TileRef) * tl.size(),
+                           cudaMemcpyHostToDevice, st));
+    I.obs_ntiles = (int)tl.size();
+    I.obs_tz = I.tz;
+    I.obs_taper = taper_;
     return NLC_OK;
   }
 
@@ -1150,13 +1206,17 @@ class Engine final : public EngineBase {
     const int64_t S = (int64_t)(Q + 5) * n;
     if ((s = ensure_unfused(I))) return s;  // Pi for the loss seed
     if (!I.lQP) {
-      if ((s = alloc(&I.lQ[0], (size_t)5 * n)) || (s = alloc(&I.lQ[1], (size_t)5 * n)) ||
-          (s = alloc(&I.lG[0], (size_t)Q * n)) || (s = alloc(&I.lG[1], (size_t)Q * n)) ||
-          (s = alloc(&I.lQP, (size_t)5 * n)) || (s = alloc(&I.lUa, (size_t)DIM * n)) ||
-          (s = alloc(&I.lGv, (size_t)DIM * DIM * n)) || (s = alloc(&I.lF, (size_t)DIM * n)) ||
-          (s = alloc(&I.lDq, (size_t)DIM * 5 * n)) || (s = alloc(&I.lLap, (size_t)5 * n)) ||
-          (s = alloc(&I.acc, (size_t)3 * (3 * grid1(n) + seg_grid_max()))))
-        return s;
+      Group mem(*this);
+      T* w[10];
+      const int64_t words[10] = {5, 5, Q, Q, 5, DIM, DIM * DIM, DIM, DIM * 5, 5};
+      double* acc = nullptr;
+      for (int k = 0; k < 10; k++)
+        if ((s = mem.alloc(&w[k], (size_t)(words[k] * n)))) return s;
+      if ((s = mem.alloc(&acc, (size_t)3 * (3 * grid1(n) + seg_grid_max())))) return s;
+      mem.kept = true;
+      I.lQ[0] = w[0], I.lQ[1] = w[1], I.lG[0] = w[2], I.lG[1] = w[3];
+      I.lQP = w[4], I.lUa = w[5], I.lGv = w[6], I.lF = w[7], I.lDq = w[8], I.lLap = w[9];
+      I.acc = acc;
     }
     if (I.ck_count < ck_count) {
       if ((s = alloc(&I.ck, (size_t)(ck_count * S)))) return s;
@@ -1532,7 +1592,13 @@ class Engine final : public EngineBase {
 
   EngineArgs args_;
   std::vector<InstHost<T, G>> inst_;
-  std::vector<void*> allocs_;
+  struct Block {
+    void* ptr;
+    size_t bytes;
+  };
+  std::vector<Block> allocs_;
+  size_t held_ = 0;                       // bytes of allocs_
+  size_t limit_ = (size_t)-1;             // of held_ (NLC_ALLOC_LIMIT)
   InstDev<T, G>* insts_dev_ = nullptr;
   CUtensorMap* qmaps_dev_ = nullptr;
   CUtensorMap* umaps_dev_ = nullptr;

@@ -94,6 +94,7 @@ struct InstHost {
   T* pi = nullptr;
   Field<T> qp;
   T* r1 = nullptr;
+  bool lent = false;  // pi, qp, r1: only the float64 cell kernels have wanted them
   T* raw = nullptr;
   double* stage = nullptr;
   double* fstage = nullptr;
@@ -288,32 +289,24 @@ class Engine final : public EngineBase {
       if (c <= maxz) cand.push_back({c, false});
     for (int c : tap)
       if (c <= maxz) cand.push_back({c, true});
+    // the cell kernels' workspaces before the saved state, whose copies must
+    // not be what keeps them out
+    nlc_status s = ensure_cells();
+    if (s) return s;
     // saved state
     const int cur0 = cur_;
     std::vector<G*> gsave(inst_.size(), nullptr);
     std::vector<T*> qsave(inst_.size(), nullptr);
-    auto release = [&]() {
-      for (G* p : gsave) cudaFree(p);
-      for (T* p : qsave) cudaFree(p);
-    };
+    Group saved(*this);
     for (size_t i = 0; i < inst_.size(); i++) {
       InstHost<T, G>& I = inst_[i];
-      const size_t gb = sizeof(G) * Q * I.d.n, qb = sizeof(T) * 5 * I.L.comp;
-      if (cudaMalloc(&gsave[i], gb) != cudaSuccess || cudaMalloc(&qsave[i], qb) != cudaSuccess) {
-        cudaGetLastError();
-        release();
-        err = "nlc_autotune: no device memory for the saved state";
-        return NLC_ENOMEM;
-      }
-      cudaMemcpyAsync(gsave[i], I.g[cur0], gb, cudaMemcpyDeviceToDevice, st);
-      cudaMemcpyAsync(qsave[i], I.q[cur0].base, qb, cudaMemcpyDeviceToDevice, st);
+      const size_t gw = (size_t)Q * I.d.n, qw = (size_t)5 * I.L.comp;
+      if ((s = saved.alloc(&gsave[i], gw)) || (s = saved.alloc(&qsave[i], qw))) return s;
+      NLC_CK(cudaMemcpyAsync(gsave[i], I.g[cur0], sizeof(G) * gw, cudaMemcpyDeviceToDevice, st));
+      NLC_CK(cudaMemcpyAsync(qsave[i], I.q[cur0].base, sizeof(T) * qw, cudaMemcpyDeviceToDevice,
+                             st));
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    nlc_status s = ensure_cells();
-    if (s) {
-      release();
-      return s;
-    }
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
       err = "nlc_autotune: cudaEventCreate failed";
       s = NLC_ECUDA;
@@ -362,7 +355,7 @@ class Engine final : public EngineBase {
                       cudaMemcpyDeviceToDevice, st);
     }
     const cudaError_t ce = cudaStreamSynchronize(st);
-    release();
+    saved.drop();
     if (s) return s;
     if (ce != cudaSuccess) {
       err = std::string("nlc_autotune: ") + cudaGetErrorString(ce);
@@ -370,6 +363,7 @@ class Engine final : public EngineBase {
     }
     if ((s = device_error())) return s;
     if ((s = set_chunk(cand[best_k].first, cand[best_k].second))) return s;
+    if ((s = retry_cells())) return s;  // had they made room for the saved state
     out->best_ms = best;
     out->chunk = 1;
     for (const auto& I : inst_) out->chunk = std::max(out->chunk, I.tz);
@@ -487,6 +481,7 @@ class Engine final : public EngineBase {
     // workspaces, the persistent kernel's occupancy and counters are set up
     // here, not inside a stream capture (no allocation may happen there)
     if ((s = ensure_cells())) return s;
+    if (kCell && !cells_captured_ && cells_dev_) cells_captured_ = capturing();
     if (persistent_steps > 0 && !any_mrt_) {
       int grid;
       if ((s = persist_grid(&grid))) return s;
@@ -596,7 +591,7 @@ class Engine final : public EngineBase {
   nlc_status set_fields_f32(int i, const float* Q5) override {
     InstHost<T, G>& I = inst_[i];
     nlc_status s;
-    if ((s = ensure_staging(I)) || (s = ensure_cells())) return s;
+    if ((s = ensure_staging(I)) || (s = retry_cells())) return s;
     const int64_t n = I.d.n;
     cudaStream_t st = args_.stream;
     // device arrays are read in place too (a caller that uploads the next
@@ -627,7 +622,7 @@ class Engine final : public EngineBase {
                         const double* u) override {
     InstHost<T, G>& I = inst_[i];
     nlc_status s;
-    if ((s = ensure_staging(I)) || (s = ensure_cells())) return s;
+    if ((s = ensure_staging(I)) || (s = retry_cells())) return s;
     const int64_t n = I.d.n;
     cudaStream_t st = args_.stream;
     // pinned inputs are read in place by the kernel (the transfer then
@@ -739,7 +734,7 @@ class Engine final : public EngineBase {
     }
     NLC_CK(cudaStreamSynchronize(st));
     cur_ = 0;
-    return ensure_cells();
+    return retry_cells();
   }
 
 
@@ -917,6 +912,14 @@ class Engine final : public EngineBase {
   template <class U>
   nlc_status alloc(U** p, size_t count) {
     const size_t bytes = sizeof(U) * (count ? count : 1);
+    void* ptr = nullptr;
+    nlc_status s = take(&ptr, bytes);
+    if (s == NLC_ENOMEM && give_back_cells()) s = take(&ptr, bytes);
+    if (!s) *p = (U*)ptr;
+    return s;
+  }
+
+  nlc_status take(void** p, size_t bytes) {
     if (bytes > limit_ - held_) {
       err = "device memory limit of the context: needs " + std::to_string(held_ + bytes) + " bytes";
       return NLC_ENOMEM;
@@ -931,7 +934,7 @@ class Engine final : public EngineBase {
     }
     allocs_.push_back({ptr, bytes});
     held_ += bytes;
-    *p = (U*)ptr;
+    *p = ptr;
     return NLC_OK;
   }
 
@@ -955,8 +958,11 @@ class Engine final : public EngineBase {
     bool kept = false;
     explicit Group(Engine& eng) : e(eng) {}
     ~Group() {
-      if (!kept)
-        for (void* p : own) e.release(p);
+      if (!kept) drop();
+    }
+    void drop() {
+      for (void* p : own) e.release(p);
+      own.clear();
     }
     template <class U>
     nlc_status alloc(U** p, size_t count) {
@@ -1023,7 +1029,9 @@ class Engine final : public EngineBase {
     return NLC_OK;
   }
 
-  nlc_status ensure_unfused(InstHost<T, G>& I) {
+  // for_cells: wanted by the cell kernels only, which can do without
+  nlc_status ensure_unfused(InstHost<T, G>& I, bool for_cells = false) {
+    I.lent = I.lent && for_cells;
     if (I.pi) return NLC_OK;
     nlc_status s;
     const int64_t n = I.d.n;
@@ -1036,40 +1044,99 @@ class Engine final : public EngineBase {
     I.pi = pi;
     I.qp = Field<T>{qp, I.L};
     I.r1 = r1;
+    I.lent = for_cells;
     return NLC_OK;
   }
 
+  // pi, qp and r1 of lattice I given back
+  void drop_unfused(InstHost<T, G>& I) {
+    release(I.pi);
+    release(I.qp.base);
+    release(I.r1);
+    I.pi = I.r1 = nullptr;
+    I.qp = Field<T>{};
+    I.lent = false;
+  }
+
   // float64 arithmetic: the workspaces (those of the unfused schedule) and
-  // descriptors of the cell kernels.  Where the workspaces do not fit on the
-  // device (set_fields and read-back need them too, so only for a context
-  // that is filled by load_state), the steps keep the tiled kernels, which
-  // need none.
+  // descriptors of the cell kernels.  Where they do not fit on the device, the
+  // steps keep the tiled kernels, which need none, until the state is next
+  // set (set_fields and read-back need the workspaces too, so that happens
+  // only to a context that is filled by load_state).
   nlc_status ensure_cells() {
     if constexpr (kCell) {
       if (cells_off_ || (cells_dev_ && !cells_stale_)) return NLC_OK;
       // nothing may be allocated or waited for inside a caller's stream
       // capture: such a step takes the tiled kernels (set_fields, load_state
       // and the calls that change the descriptors build them beforehand)
-      // (the query itself fails on the legacy stream while another stream is
-      // being captured)
-      cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-      if (cudaStreamIsCapturing(args_.stream, &capturing) != cudaSuccess) {
+      if (capturing()) return NLC_OK;
+      std::vector<InstHost<T, G>*> made;
+      building_cells_ = true;
+      const nlc_status s = build_cells(&made);
+      building_cells_ = false;
+      if (!s) return s;
+      for (InstHost<T, G>* I : made) drop_unfused(*I);
+      if (s != NLC_ENOMEM) return s;
+      cells_off_ = true;
+      err.clear();
+    }
+    return NLC_OK;
+  }
+
+  // the same where the state is set, after an earlier lack of memory too
+  nlc_status retry_cells() {
+    cells_off_ = false;
+    return ensure_cells();
+  }
+
+  // the context's stream is being captured, or (the query fails) is the legacy
+  // stream while another is
+  bool capturing() {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(args_.stream, &c) != cudaSuccess) {
+      cudaGetLastError();
+      return true;
+    }
+    return c != cudaStreamCaptureStatusNone;
+  }
+
+  // Returns the workspaces that only the cell kernels have wanted, for an
+  // allocation that would not fit beside them; the steps go on with the tiled
+  // kernels.  Not while a caller's graph may hold them.  True: there is more
+  // memory now.
+  bool give_back_cells() {
+    if constexpr (kCell) {
+      if (building_cells_ || cells_captured_ || !cells_dev_) return false;
+      bool any = false;
+      for (auto& I : inst_) any = any || I.lent;
+      if (!any || cudaStreamSynchronize(args_.stream) != cudaSuccess) {
         cudaGetLastError();
-        return NLC_OK;
+        return false;
       }
-      if (capturing != cudaStreamCaptureStatusNone) return NLC_OK;
+      drop_graphs();
+      for (auto& I : inst_)
+        if (I.lent) drop_unfused(I);
+      cells_off_ = cells_stale_ = true;
+      return true;
+    }
+    return false;
+  }
+
+  // workspaces (the lattices that got theirs here go to *made), descriptors
+  nlc_status build_cells(std::vector<InstHost<T, G>*>* made) {
+    if constexpr (kCell) {
       nlc_status s;
       const size_t n = inst_.size();
-      for (size_t i = 0; i < n; i++) {
-        s = ensure_unfused(inst_[i]);
-        if (s == NLC_ENOMEM) {
-          cells_off_ = true;
-          err.clear();
-          return NLC_OK;
-        }
-        if (s) return s;
+      int64_t blocks = 0;
+      for (auto& I : inst_) blocks += (I.d.n + CELL_T - 1) / CELL_T;
+      if (blocks > INT32_MAX) return NLC_ENOMEM;
+      for (auto& I : inst_) {
+        if (I.pi) continue;
+        if ((s = ensure_unfused(I, true))) return s;
+        made->push_back(&I);
       }
-      if (!cells_dev_ && (s = alloc(&cells_dev_, 2 * n))) return s;
+      const bool fresh = !cells_dev_;
+      if (fresh && (s = alloc(&cells_dev_, 2 * n))) return s;
       if (any_mrt_ && !cell_mrt_ && (s = alloc(&cell_mrt_, n * Q))) return s;
       std::vector<CellInst<G>> ci(2 * n);
       std::vector<double> rates(n * Q, 0.0);
@@ -1096,10 +1163,6 @@ class Engine final : public EngineBase {
         ci[n + i] = C;
         ci[n + i].c = make_cell_par<Lat>(I.p, true);
       }
-      if (nb > INT32_MAX) {
-        cells_off_ = true;
-        return NLC_OK;
-      }
       cell_blocks_ = (unsigned)nb;
       cudaStream_t st = args_.stream;
       if (any_mrt_)
@@ -1109,6 +1172,7 @@ class Engine final : public EngineBase {
                              cudaMemcpyHostToDevice, st));
       NLC_CK(cudaStreamSynchronize(st));
       cells_stale_ = false;
+      if (!made->empty() || fresh) drop_graphs();  // they hold tiled steps
     }
     return NLC_OK;
   }
@@ -1617,6 +1681,8 @@ class Engine final : public EngineBase {
   unsigned cell_blocks_ = 0;
   bool cells_stale_ = true;      // to be uploaded before the next step
   bool cells_off_ = false;       // workspaces do not fit: tiled kernels
+  bool cells_captured_ = false;  // a caller's graph may hold the workspaces
+  bool building_cells_ = false;
   unsigned long long* bad_ = nullptr;
   unsigned* derr_ = nullptr;
   int cur_ = 0;

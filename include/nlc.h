@@ -289,7 +289,9 @@ NLC_API int32_t nlc_get_chunk(const nlc_ctx* ctx, int32_t inst, int32_t* taper);
  * object keyed by lattice, precision, extents, collision, stencils and GPU
  * (name, SM count), with the chunk depth as value (negative for a tapered
  * list): a key found there is applied without timing (out->from_cache = 1),
- * a new result is added.  Needs two extra copies of the populations and Q of the whole
+ * a new result is added.  In float64 arithmetic, whose kernels do not use the
+ * list, only the default is timed (candidates = 1) and no result is added.
+ * Needs two extra copies of the populations and Q of the whole
  * context in device memory while it runs (freed before it returns).  out may
  * be NULL.  Synchronises the stream.
  * Errors: NLC_EINVAL (trial_steps < 1), NLC_ENOMEM, NLC_ECUDA,

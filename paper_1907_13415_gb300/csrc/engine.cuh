@@ -263,6 +263,7 @@ class Engine final : public EngineBase {
   }
 
   int chunk(int i) const override { return inst_[i].tz; }
+  bool uses_chunks() const override { return !cells_active(); }
   bool tapered() const override { return taper_; }
 
   // Candidate depths are timed on the current state, which is saved first
@@ -306,6 +307,8 @@ class Engine final : public EngineBase {
       NLC_CK(cudaMemcpyAsync(qsave[i], I.q[cur0].base, sizeof(T) * qw, cudaMemcpyDeviceToDevice,
                              st));
     }
+    // the cell kernels do not read the list: there is nothing to choose
+    if (cells_active()) cand.resize(1);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
       err = "nlc_autotune: cudaEventCreate failed";
@@ -1065,7 +1068,7 @@ class Engine final : public EngineBase {
   // only to a context that is filled by load_state).
   nlc_status ensure_cells() {
     if constexpr (kCell) {
-      if (cells_off_ || (cells_dev_ && !cells_stale_)) return NLC_OK;
+      if (cells_off_ || cells_active()) return NLC_OK;
       // nothing may be allocated or waited for inside a caller's stream
       // capture: such a step takes the tiled kernels (set_fields, load_state
       // and the calls that change the descriptors build them beforehand)
@@ -1082,6 +1085,9 @@ class Engine final : public EngineBase {
     }
     return NLC_OK;
   }
+
+  // steps run as the cell kernels
+  bool cells_active() const { return cells_dev_ && !cells_off_ && !cells_stale_; }
 
   // the same where the state is set, after an earlier lack of memory too
   nlc_status retry_cells() {
@@ -1551,7 +1557,7 @@ class Engine final : public EngineBase {
 
   // one step of every lattice: two launches over the joint tile list
   nlc_status step_fused(cudaStream_t st) {
-    if (cells_dev_ && !cells_off_ && !cells_stale_) return step_cells(st);
+    if (cells_active()) return step_cells(st);
     const int a = cur_;
     const int e0 = mark();
     cudaError_t e = launch_fused_lb<Lat, T>(insts_dev_, qmaps_dev_, tiles_dev_, ntiles_, a,

@@ -92,6 +92,8 @@ struct EngineBase {
   // taper: the last chunks of every column shrink (chunk_bounds)
   virtual nlc_status set_chunk(int tz, bool taper) = 0;
   virtual int chunk(int inst) const = 0;
+  // whether the steps read the chunk list (the float64 cell kernels do not)
+  virtual bool uses_chunks() const = 0;
   virtual bool tapered() const = 0;
   // times `trial_steps` fused steps for each candidate chunk depth on the
   // current state, restores the state and keeps the fastest depth

@@ -282,7 +282,7 @@ nlc_status nlc_autotune(nlc_ctx* ctx, int32_t trial_steps, nlc_tune* out) {
   } else {
     if ((st = ctx->eng->autotune(trial_steps, &res)) != NLC_OK)
       return fail(ctx, st, ctx->eng->err);
-    if (!path.empty() &&
+    if (!path.empty() && ctx->eng->uses_chunks() &&
         !nlc::tune_cache_put(path, key, res.taper ? -(long)res.chunk : (long)res.chunk))
       return fail(ctx, NLC_EINVAL, "nlc_autotune: cannot write the cache file " + path);
   }

@@ -243,12 +243,14 @@ class Engine final : public EngineBase {
       append_tiles<Lat>((int)i, I.d, z, taper, &tiles);
     }
     NLC_CK(cudaStreamSynchronize(st));  // no step may still read the old list
-    if (tiles.size() > tiles_cap_) {
-      // the old list stays until there is a new one
+    // a list that a caller's graph holds stays as it is; others are reused, or
+    // given back once there is a longer one
+    if (tiles.size() > tiles_cap_ || captured_) {
       TileRef* list = nullptr;
       nlc_status s = alloc(&list, tiles.size());
       if (s) return s;
-      release(tiles_dev_);
+      if (!captured_) release(tiles_dev_);
+      captured_ = false;
       tiles_dev_ = list;
       tiles_cap_ = tiles.size();
     }
@@ -484,7 +486,10 @@ class Engine final : public EngineBase {
     // workspaces, the persistent kernel's occupancy and counters are set up
     // here, not inside a stream capture (no allocation may happen there)
     if ((s = ensure_cells())) return s;
-    if (kCell && !cells_captured_ && cells_dev_) cells_captured_ = capturing();
+    if ((!captured_ || (kCell && !cells_captured_)) && capturing()) {
+      captured_ = true;
+      cells_captured_ = cells_captured_ || cells_active();
+    }
     if (persistent_steps > 0 && !any_mrt_) {
       int grid;
       if ((s = persist_grid(&grid))) return s;
@@ -1674,6 +1679,7 @@ class Engine final : public EngineBase {
   CUtensorMap* umaps_dev_ = nullptr;
   TileRef* tiles_dev_ = nullptr;
   size_t tiles_cap_ = 0;
+  bool captured_ = false;  // a caller's graph may hold this list
   bool taper_ = false;  // tapered chunk lists (chunk_bounds)
   int ntiles_ = 0;
   bool maps_ok_ = false;

@@ -68,3 +68,35 @@ def test_replay_after_a_change(name, precision):
     assert np.array_equal(a.get_fields()[0], b.get_fields()[0])
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("lattice", [wl.D2Q9, wl.D3Q19], ids=["d2q9", "d3q19"])
+def test_replay_after_other_chunk_lists(lattice):
+    """A captured graph keeps its chunk list, whatever lists are set later."""
+    import torch
+    from paper_1907_13415_gb300 import nlc
+    shape = (1, 61, 70) if lattice == wl.D2Q9 else (23, 20, 40)
+    base = wl.disc_256() if lattice == wl.D2Q9 else wl.sphere_256()
+    w = base.with_(lattice=lattice, shape=shape, size=6.0, noise=1e-3, seed=SEED)
+    stream = torch.cuda.Stream()
+    out = []
+    for captured in (False, True):
+        s = nlc.Simulation(lattice, shape, w.params, precision=nlc.NLC_FP32,
+                           stream=stream.cuda_stream)
+        s.set_fields(w.initial_q5())
+        if captured:
+            s.set_chunk(4, True)
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=stream):
+                s.step(2)
+            for chunk in (64, 1, 3):  # shorter, longer, in between
+                s.set_chunk(chunk)
+                with torch.cuda.stream(stream):
+                    g.replay()
+                s.step(2)
+        else:
+            s.step(12)
+        out.append((s.get_populations(), s.get_fields()[0]))
+        s.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)

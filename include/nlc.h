@@ -264,7 +264,9 @@ NLC_API nlc_status nlc_set_schedule(nlc_ctx* ctx, int32_t schedule);
  * stacked along y, loading the next tile while it computes the current one;
  * the depth counts those tiles.  chunk > 0: chunks of that many planes
  * (tiles), capped at the column's length; chunk = 0: the library's default
- * depth.  taper = 1: chunks of `chunk` until at most 2 chunk of the column
+ * depth, which for one float32 D3Q19 lattice may differ between the stencils
+ * and for the persistent form (a change of those rebuilds the list then, and
+ * synchronises the stream, unless that is being captured).  taper = 1: chunks of `chunk` until at most 2 chunk of the column
  * remain, then chunks halving down to about 8 planes (tiles); the blocks run
  * chunk by chunk, so the last blocks are short and the last wave over the
  * SMs idles less of the GPU.  Neither changes any result: every chunk list

@@ -44,10 +44,10 @@ inline std::vector<int> chunk_bounds(int nz, int tz, bool taper) {
 // recomputes and its start) times 3.9 us when it has an SM to itself, 6.3 us
 // when one wave of blocks fills SMs twice (their phases coincide), 5.0 us in
 // several waves, where the blocks of a list start in order on the first free
-// slot.  Fitted to 13 lattices from 20 to 256 planes a side: choosing among
-// uniform and tapered lists by it came within 1.4% of the fastest on average,
-// and up to 7% on one lattice.
-inline double estimate_step_us(int nz, long columns, int tz, int sms) {
+// slot; tail_us is the time per plane once every block left has an SM to
+// itself (5.0: as before; 3.9 comes closer for a short last wave, but then
+// the other constants, fitted without it, favour other depths).
+inline double estimate_step_us(int nz, long columns, int tz, int sms, double tail_us = 5.0) {
   const double extra = 1.5;
   const std::vector<int> b = chunk_bounds(nz, tz, false);
   const long blocks = columns * (long)(b.size() - 1);
@@ -68,7 +68,14 @@ inline double estimate_step_us(int nz, long columns, int tz, int sms) {
       n -= m;
     }
   }
-  return 5.0 * free_at.rbegin()->first;
+  double alone = 0.0, t = 0.0;  // planes during which no SM has two blocks
+  long busy = 2L * sms;
+  for (const auto& e : free_at) {
+    if (busy <= sms) alone += e.first - t;
+    busy -= e.second;
+    t = e.first;
+  }
+  return 5.0 * t - (5.0 - tail_us) * alone;
 }
 
 // Uniform depth with the smallest estimate, or `fallback` unless that is
@@ -85,6 +92,54 @@ inline int estimated_depth(int nz, long columns, int sms, int fallback) {
       tz = c;
     }
   }
+  return tz;
+}
+
+// Planes (plus 1.5 per tile) of the busiest of `blocks` blocks that take the
+// tiles of such a list in turn, as the persistent kernel's do.
+inline double round_robin_planes(int nz, long columns, int tz, long blocks) {
+  const std::vector<int> b = chunk_bounds(nz, tz, false);
+  std::vector<double> planes((size_t)blocks, 0.0);
+  double worst = 0.0;
+  long tile = 0;
+  for (size_t k = 0; k + 1 < b.size(); k++)
+    for (long c = 0; c < columns; c++, tile++) {
+      double& mine = planes[(size_t)(tile % blocks)];
+      mine += b[k + 1] - b[k] + 1.5;
+      worst = mine > worst ? mine : worst;
+    }
+  return worst;
+}
+
+// How the steps of a context run, as far as the default depth depends on it.
+struct StepForm {
+  bool isotropic, persistent;
+};
+
+// Default depth of one FP32 D3Q19 lattice: estimated_depth, which was fitted
+// to the two step kernels with the standard stencils (BGK and MRT alike),
+// unless the form of the step makes `fallback` the better choice:
+//   - isotropic stencils: where the estimate with a cheaper last wave does not
+//     see the tenth (51 x 67 x 90 82 us at that depth, 77 at the fallback;
+//     48 x 175 x 34 81 / 76; 198 x 59 x 137 271 / 295, which stays);
+//   - persistent kernel: where some blocks have several tiles and the busiest
+//     gets no less to do (70 x 180 x 50 105 us, fallback 98; 100^3 137 / 160,
+//     which stays).
+// Over 48 lattices of 20 to 200 planes a side, time at the fallback over time
+// at the default, geometric mean and worst: standard 1.10, 0.96; MRT 1.10,
+// 0.97; isotropic 1.10, 1.00 (0.94 without the check); persistent 1.14, 0.98
+// (0.93).
+inline int default_depth(int nz, long columns, int sms, int fallback, StepForm form) {
+  const int tz = estimated_depth(nz, columns, sms, fallback);
+  if (tz == fallback) return tz;
+  if (form.isotropic && estimate_step_us(nz, columns, tz, sms, 3.9) >
+                            0.9 * estimate_step_us(nz, columns, fallback, sms, 3.9))
+    return fallback;
+  const long tiles = columns * (long)(chunk_bounds(nz, tz, false).size() - 1);
+  if (form.persistent && tiles > 2L * sms &&
+      round_robin_planes(nz, columns, tz, 2L * sms) >=
+          round_robin_planes(nz, columns, fallback, 2L * sms))
+    return fallback;
   return tz;
 }
 

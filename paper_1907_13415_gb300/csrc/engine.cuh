@@ -230,16 +230,7 @@ class Engine final : public EngineBase {
       int& z = depth[i];
       z = tz > 0 ? std::min(tz, column_length<Lat>(I.d))
                  : fused_tz<Lat>(I.d, (int64_t)tiles.size());
-      if (tz <= 0 && DIM == 3 && !kCell && inst_.size() == 1) {
-        // the estimate covers one float32 D3Q19 lattice with the device to
-        // itself (us per step at its depth / the rule above: 128^3 177 / 199,
-        // 160^3 319 / 326, 70 x 180 x 50 80 / 91, 32^3 16 / 24)
-        int dev = 0, sms = 0;
-        NLC_CK(cudaGetDevice(&dev));
-        NLC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        const long columns = (long)((I.d.nx + FTX - 1) / FTX) * ((I.d.ny + FTY - 1) / FTY);
-        z = estimated_depth(I.d.nz, columns, sms, z);
-      }
+      if (tz <= 0 && !taper) NLC_CK(estimate_depth(&z));
       append_tiles<Lat>((int)i, I.d, z, taper, &tiles);
     }
     NLC_CK(cudaStreamSynchronize(st));  // no step may still read the old list
@@ -255,6 +246,7 @@ class Engine final : public EngineBase {
       tiles_cap_ = tiles.size();
     }
     taper_ = taper;
+    default_list_ = tz <= 0 && !taper;
     for (size_t i = 0; i < inst_.size(); i++) inst_[i].tz = depth[i];
     ntiles_ = (int)tiles.size();
     NLC_CK(cudaMemcpyAsync(tiles_dev_, tiles.data(), sizeof(TileRef) * tiles.size(),
@@ -262,6 +254,34 @@ class Engine final : public EngineBase {
     NLC_CK(cudaStreamSynchronize(st));
     drop_graphs();
     return NLC_OK;
+  }
+
+  // *z: default depth of the lattice by the rule that knows nothing of the
+  // step's form; replaced by the estimate for what it covers, one float32
+  // D3Q19 lattice with the device to itself and a uniform list (us per step at
+  // its depth / the rule's: 128^3 176 / 199, 160^3 316 / 324, 70 x 180 x 50
+  // 79 / 90, 32^3 12 / 23)
+  cudaError_t estimate_depth(int* z) {
+    if (DIM != 3 || kCell || inst_.size() != 1) return cudaSuccess;
+    const Dims& d = inst_[0].d;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const long columns = (long)((d.nx + FTX - 1) / FTX) * ((d.ny + FTY - 1) / FTY);
+    *z = default_depth(d.nz, columns, sms, *z, StepForm{iso_, persistent_steps > 0});
+    return cudaSuccess;
+  }
+
+  // The default list follows the step's form.  Not inside a stream capture,
+  // and where there is no room for the other list this one stays.
+  nlc_status form_changed() override {
+    if (DIM != 3 || !default_list_) return NLC_OK;
+    int z = fused_tz<Lat>(inst_[0].d, 0);
+    NLC_CK(estimate_depth(&z));
+    if (inst_.size() != 1 || z == inst_[0].tz || capturing()) return NLC_OK;
+    const nlc_status s = set_chunk(0, false);
+    return s == NLC_ENOMEM ? NLC_OK : s;
   }
 
   int chunk(int i) const override { return inst_[i].tz; }
@@ -442,9 +462,10 @@ class Engine final : public EngineBase {
 
   // stencils of every lattice: standard (false) or isotropic (true)
   nlc_status set_stencil(bool iso) override {
-    if (iso != iso_) drop_graphs();
+    if (iso == iso_) return NLC_OK;
+    drop_graphs();
     iso_ = iso;
-    return NLC_OK;
+    return form_changed();
   }
 
   nlc_status set_params(int i, const nlc_params& q) override {
@@ -1680,6 +1701,7 @@ class Engine final : public EngineBase {
   TileRef* tiles_dev_ = nullptr;
   size_t tiles_cap_ = 0;
   bool captured_ = false;  // a caller's graph may hold this list
+  bool default_list_ = false;  // of the default depth
   bool taper_ = false;  // tapered chunk lists (chunk_bounds)
   int ntiles_ = 0;
   bool maps_ok_ = false;

@@ -95,6 +95,8 @@ struct EngineBase {
   // whether the steps read the chunk list (the float64 cell kernels do not)
   virtual bool uses_chunks() const = 0;
   virtual bool tapered() const = 0;
+  // after a change of what the default depth depends on (persistent_steps)
+  virtual nlc_status form_changed() = 0;
   // times `trial_steps` fused steps for each candidate chunk depth on the
   // current state, restores the state and keeps the fastest depth
   virtual nlc_status autotune(int trial_steps, nlc_tune* out) = 0;

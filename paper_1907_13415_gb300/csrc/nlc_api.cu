@@ -207,7 +207,10 @@ nlc_status nlc_set_persistent(nlc_ctx* ctx, int32_t steps) {
   if (!ctx) return NLC_EINVAL;
   if (steps < 0) return fail(ctx, NLC_EINVAL, "negative persistent step count");
   if (steps != ctx->eng->persistent_steps) ctx->eng->invalidate_graphs();
+  const bool changed = (steps > 0) != (ctx->eng->persistent_steps > 0);
   ctx->eng->persistent_steps = steps;
+  nlc_status st = changed ? ctx->eng->form_changed() : NLC_OK;
+  if (st != NLC_OK) return fail(ctx, st, ctx->eng->err);
   return NLC_OK;
 }
 

@@ -51,10 +51,21 @@ PRECISIONS = {"fp32": ("NLC_FP32", 4, 4, "f32"),
 
 
 def alg_bytes(precision):
-    """(step, per-kernel) algorithmic bytes per LUP for a precision."""
-    _, gw, qw, _ = PRECISIONS[precision]
-    return (2 * (Q3 * gw + 5 * qw),
-            {"fused_lb": 2 * Q3 * gw + 5 * qw, "fused_be": 2 * 5 * qw})
+    """(step, per-kernel) algorithmic bytes per LUP for a precision.  Float64
+    arithmetic runs four kernels, which share the bytes out: stress and
+    predict read Q, lb reads and writes the populations, correct writes Q (they
+    are bound by the float64 instruction rate, not by these)."""
+    _, gw, qw, arith = PRECISIONS[precision]
+    step = 2 * (Q3 * gw + 5 * qw)
+    if arith == "f64":
+        return step, {"stress": 5 * qw, "lb": 2 * Q3 * gw, "predict": 5 * qw, "correct": 5 * qw}
+    return step, {"fused_lb": 2 * Q3 * gw + 5 * qw, "fused_be": 2 * 5 * qw}
+
+
+def step_label(kernels):
+    """The step, named by the kernels that ran in it."""
+    return "step (" + " + ".join(kernels) + ")"
+
 
 # DRAM traffic per LUP of each kernel from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum, divided by the cells of the
@@ -479,8 +490,8 @@ def run_ours(args, w):
     value, t_max = whole_job_rate(cells, args.steps, elapsed_ms, ws)
     launches = sum(n for _, n in kt.values())
 
-    # roofline of the step (the pair of fused kernels that makes one time
-    # step): algorithmic bytes 2 (q + 5) words per lattice update over the
+    # roofline of the step (the kernels that make one time step):
+    # algorithmic bytes 2 (q + 5) words per lattice update over the
     # device time of a step, against the measured HBM copy bandwidth; the
     # per-kernel figures sit under "kernels"
     peak, peak_src = hbm_peak()
@@ -510,7 +521,7 @@ def run_ours(args, w):
     achieved = step_bytes * cells / step_s / 1e9
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "traffic": step_traffic,
-                "kernel": "step (fused_lb + fused_be)", "peak_source": peak_src,
+                "kernel": step_label(kernels), "peak_source": peak_src,
                 "alg_bytes_per_lup": step_bytes,
                 "numerator": (f"{step_bytes} B/LUP x {cells} cells (read + write of the "
                               f"{Q3} populations and 5 Q components) / device time of "

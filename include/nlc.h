@@ -78,8 +78,11 @@ enum {
 
 /* Kernel schedule of one step.  Both compute the same step. */
 enum {
-  NLC_SCHED_FUSED = 0,  /* two tiled kernels per step (default)            */
-  NLC_SCHED_UNFUSED = 1 /* four one-cell-per-thread kernels per step        */
+  NLC_SCHED_FUSED = 0,  /* default: two tiled kernels per step, in float64
+                           arithmetic four one-cell-per-thread kernels (see
+                           nlc_step)                                       */
+  NLC_SCHED_UNFUSED = 1 /* four one-cell-per-thread kernels per step and
+                           lattice, in the plain form of the equations     */
 };
 
 typedef struct {
@@ -189,7 +192,8 @@ NLC_API nlc_status nlc_set_graph(nlc_ctx* ctx, int32_t steps);
  * the two-kernel form bit for bit.  Combines with nlc_set_graph (a graph
  * then holds the cooperative launches).  0 (default): two kernel launches
  * per step.  The MRT collision, float64 arithmetic (NLC_FP64, NLC_FP32_QF64)
- * and devices without cooperative launch keep the form of separate kernels.  Errors: NLC_EINVAL (steps < 0). */
+ * and devices without cooperative launch keep the form of separate kernels.
+ * Errors: NLC_EINVAL (steps < 0), NLC_ECUDA. */
 NLC_API nlc_status nlc_set_persistent(nlc_ctx* ctx, int32_t steps);
 
 /* Finite-difference stencils of the context (every lattice).
@@ -202,7 +206,8 @@ NLC_API nlc_status nlc_set_persistent(nlc_ctx* ctx, int32_t steps);
  * names for the spurious currents.  Applies to every derivative of the
  * step (grad Q, lap Q, grad u, div Pi) and to the force in the observables;
  * nlc_observables_static keeps the standard stencils.  nlc_adjoint returns
- * NLC_EUNSUPPORTED with the isotropic stencils.  Errors: NLC_EINVAL. */
+ * NLC_EUNSUPPORTED with the isotropic stencils.  Errors: NLC_EINVAL,
+ * NLC_ECUDA. */
 #define NLC_STENCIL_STANDARD 0
 #define NLC_STENCIL_ISOTROPIC 1
 NLC_API nlc_status nlc_set_stencil(nlc_ctx* ctx, int32_t kind);
@@ -376,7 +381,9 @@ NLC_API nlc_status nlc_load(nlc_ctx* ctx, const void* buf, size_t len);
 /* Per-kernel device timing (CUDA events recorded on the context's stream
  * around each kernel launch of nlc_step).  enable = 1 clears the log and
  * starts recording; enable = 0 stops.  Meant for profiling: while enabled,
- * each step records one extra event per kernel. */
+ * each step records one extra event per kernel.  The fused schedule reports
+ * fused_lb and fused_be (or fused_persistent), in float64 arithmetic stress, lb,
+ * predict and correct, as the unfused schedule does. */
 NLC_API nlc_status nlc_set_timing(nlc_ctx* ctx, int32_t enable);
 
 /* Totals since timing was enabled, per kernel id (0 .. NLC_N_KERNELS-1):

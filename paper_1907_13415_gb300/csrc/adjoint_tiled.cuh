@@ -14,10 +14,11 @@
 // through global memory, so one grid barrier per reverse step remains.
 // A box cell's halo values are recomputed by every block whose box holds
 // it; each block writes global adjoints and adds parameter adjoints for its
-// own tile only.  Every cell value is formed by the same functions in the
-// same order as in the segment kernel, so the state adjoints agree to
-// rounding (the compiler may contract multiply-adds differently in the two
-// kernels); the parameter adjoints are summed in another grouping.
+// own tile only.  The reverse stages use the functions of the segment kernel
+// (adjoint_point.cuh); the record's formulas are those of the step kernels
+// (physics.cuh: *_tl, mrt.cuh), where the segment kernel takes the plain ones.
+// So the state adjoints of the two forms agree to rounding; the parameter
+// adjoints are summed in another grouping.
 #pragma once
 #include "adjoint.cuh"
 #include "adjoint_segment.cuh"
@@ -274,10 +275,10 @@ __global__ void __maxnreg__(96) k_seg_reverse_tiled(SegArgs<T> a, int tiles_x) {
 // ---------------------------------------------------------------------------
 // record of a segment on the same tiles
 // ---------------------------------------------------------------------------
-// The forward recomputation of a segment (as k_seg_record: the stress, lb,
-// predictor and corrector stages of step_unfused.cuh, keeping Pi, u, Q^P
-// and the next state in the record slots) with the intermediates of a step
-// in shared memory on the tile's box: the stress on r <= 3, the lb update
+// The forward recomputation of a segment (the stages of k_seg_record, stress,
+// lb, predictor and corrector, keeping Pi, u, Q^P and the next state in the
+// record slots, in the formulas of the step kernels) with the intermediates
+// of a step in shared memory on the tile's box: the stress on r <= 3, the lb update
 // (u) on r <= 2, the predictor (Q^P) on r <= 1, the corrector on the tile,
 // one grid barrier per step.  Records are written for the owned cells
 // (with the periodic images of the padded fields).

@@ -45,8 +45,8 @@ inline std::vector<int> chunk_bounds(int nz, int tz, bool taper) {
 // when one wave of blocks fills SMs twice (their phases coincide), 5.0 us in
 // several waves, where the blocks of a list start in order on the first free
 // slot; tail_us is the time per plane once every block left has an SM to
-// itself (5.0: as before; 3.9 comes closer for a short last wave, but then
-// the other constants, fitted without it, favour other depths).
+// itself (5.0, which the other constants were fitted with, or 3.9, which is
+// closer for a short last wave).
 inline double estimate_step_us(int nz, long columns, int tz, int sms, double tail_us = 5.0) {
   const double extra = 1.5;
   const std::vector<int> b = chunk_bounds(nz, tz, false);

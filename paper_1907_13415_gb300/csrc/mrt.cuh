@@ -1,15 +1,16 @@
 // mrt.cuh -- the collisions of physics.cuh (collide_bgk, collide_mrt) on sums
 // and differences of opposite populations.
 //
-// The moment rows of the multiple-relaxation-time collision are even or odd under c -> -c and built from few groups of
-// velocities: the even ones see only the sum of each axis pair, and the sum
-// and difference of the two pairs of each diagonal plane; the odd ones the
-// differences along one axis.  Transforming those groups instead of the
-// populations takes about a fifth of the operations of the dense rows (D3Q19,
-// 15 rows: about 60 instead of 400), and the equilibrium and source term
-// enter each group in closed form, so no per-population copies of them are
-// kept.  Measured on the 128^3 D3Q19 lattice in FP32, k_fused_lb with this
-// collision: 184 -> 122 us (the dense rows also went through local memory, and
+// The moment rows of the multiple-relaxation-time collision are even or odd
+// under c -> -c and built from few groups of velocities: the even ones see
+// only the sum of each axis pair, and the sum and difference of the two pairs
+// of each diagonal plane; the odd ones the differences along one axis.
+// Transforming those groups instead of the populations takes about a fifth of
+// the operations of the dense rows (D3Q19, 15 rows: about 60 instead of 400),
+// and the equilibrium and source term enter each group in closed form, so no
+// per-population copies of them are kept.  Measured on the 128^3 D3Q19 lattice
+// in FP32, k_fused_lb with this collision: 184 -> 122 us at equal chunk depth
+// (105 at the present one; the dense rows also went through local memory, and
 // rounding left small non-zero entries in rows that are zero there).
 #pragma once
 #include "lattice.cuh"

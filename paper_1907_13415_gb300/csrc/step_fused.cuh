@@ -760,9 +760,8 @@ struct BeCfg {
 };
 
 // u and G2[a][b] = 2 d_b u_a (plain differences, twice the central
-// difference) at box offset o (z neighbours from the planes above and
-// below); the caller halves the factors that multiply G2, which gives the
-// same products as the gradient with its halved coefficients, exactly
+// difference, as be_rhs_tl takes them) at box offset o (z neighbours from
+// the planes above and below)
 template <class Lat, class T, bool ISO>
 __device__ __forceinline__ void box_ugrad(const T* __restrict__ c,
                                           const T* __restrict__ m,
@@ -816,8 +815,8 @@ __device__ __forceinline__ void box_ugrad(const T* __restrict__ c,
 // Q, twice the advection, u.(2 dQ) = 2 u.grad Q, and the Laplacian at
 // offset o of a plane array c (row stride row, component stride comp; z
 // neighbours in m and pp).  The differences are kept plain (twice the
-// central difference); the caller takes the advection with the factor -1/2
-// (be_rhs_adv), which is exact.
+// central difference); be_rhs_tl takes the advection with the factor -1/2,
+// which is exact.
 template <class Lat, class T, bool ISO>
 __device__ __forceinline__ void stencil_adv(const T* __restrict__ c, const T* __restrict__ m,
                                             const T* __restrict__ pp, int o, int row, int comp,
@@ -1140,7 +1139,8 @@ __global__ void __launch_bounds__(PersistCfg<Lat, T>::THREADS, PersistCfg<Lat, T
         const bool ok =
             ph == 0 ? fused_lb_tile<Lat, T, G, false, ISO, IX32, false, true>(
                           tiles[t], insts, qmaps, cur, err, nullptr, 0)
-                    : fused_be_tile<Lat, T, G, ISO, true>(tiles[t], insts, qmaps, umaps, cur, err, 0);
+                    : fused_be_tile<Lat, T, G, ISO, true>(tiles[t], insts, qmaps, umaps, cur,
+                                                          err, 0);
         if (!ok) return;
       }
       // the phase's global writes are read by TMA copies after the barrier
@@ -1237,8 +1237,8 @@ inline int resident_blocks(K kernel, int threads, size_t smem, ResidentCache& c)
 
 // A step kernel launched with programmatic stream serialisation (see
 // grid_dep_wait): it may be scheduled while the previous kernel of the
-// stream finishes, and waits for it on the device before its first global
-// access.  Inside a stream capture the dependency becomes a programmatic
+// stream finishes, and waits for it on the device before its first access to
+// memory that kernels write.  Inside a stream capture the dependency becomes a programmatic
 // edge of the graph.
 template <class... KArgs, class... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int threads, size_t smem,
@@ -1263,8 +1263,12 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int threads, s
 // of one wave keeps the form for two, which has more loads in flight per
 // thread and, started early behind the previous kernel, spreads evenly.
 // us per step, two / three blocks (FP32): 64-lattice sweep 109.5 / 94.5,
-// 512^2 20.0 / 17.3, 2035 x 1501 138 / 126, 4096^2 643 / 611; 256^2 (256
-// blocks) 6.2 / 7.8.
+// 512^2 19.7 / 17.0 (isotropic stencils 24.1 / 20.9, MRT 20.4 / 17.7),
+// 2035 x 1501 138 / 126 (183 / 168, 154 / 129), 4096^2 643 / 611; 256^2 (256
+// blocks) 6.2 / 7.8.  A launch of 305 to 456 blocks is one wave of three per SM,
+// without an early release, and no exception: 280^2 (315 blocks) 9.8 / 8.3
+// (11.4 / 10.1, 10.2 / 8.6), 320^2 (400 blocks) 10.7 / 8.6 (12.2 / 10.4,
+// 10.9 / 9.0).
 template <class Lat, class T>
 constexpr int many_blocks() {
   return Lat::DIM == 2 && sizeof(T) == 4 ? 3 : 0;
@@ -1273,9 +1277,9 @@ constexpr int many_blocks() {
 // Launches kernel2, compiled for blocks2 blocks per SM (the default), or,
 // when the launch takes more than one wave of it, kernel3 (if given).
 template <class K2, class K3, class... Args>
-cudaError_t launch_step(bool marching, K2 kernel2, int blocks2, K3 kernel3, bool have3, int threads, size_t smem, int ntiles,
-                        unsigned long long* configured, ResidentCache* resident, cudaStream_t st,
-                        Args... args) {
+cudaError_t launch_step(bool marching, K2 kernel2, int blocks2, K3 kernel3, bool have3,
+                        int threads, size_t smem, int ntiles, unsigned long long* configured,
+                        ResidentCache* resident, cudaStream_t st, Args... args) {
   cudaError_t e = set_smem(kernel2, smem, &configured[0]);
   if (e != cudaSuccess) return e;
   // The next kernel is released early.  On D3Q19, where a block marches through
@@ -1354,8 +1358,9 @@ cudaError_t launch_fused_be_as(const InstDev<T, G>* insts, const CUtensorMap* qm
   static ResidentCache resident;
   constexpr int M2 = BeCfg<Lat, T>::MINB, M3 = many_blocks<Lat, T>();
   return launch_step(Lat::DIM == 3, k_fused_be<Lat, T, G, ISO, M2>, M2,
-                     k_fused_be<Lat, T, G, ISO, M3 ? M3 : M2>, M3 != 0, BeCfg<Lat, T>::THREADS, BeCfg<Lat, T>::bytes, ntiles, configured,
-                     &resident, st, insts, qmaps, umaps, tiles, cur, err);
+                     k_fused_be<Lat, T, G, ISO, M3 ? M3 : M2>, M3 != 0,
+                     BeCfg<Lat, T>::THREADS, BeCfg<Lat, T>::bytes, ntiles, configured, &resident,
+                     st, insts, qmaps, umaps, tiles, cur, err);
 }
 
 template <class Lat, class T, class G>

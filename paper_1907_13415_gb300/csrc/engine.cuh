@@ -324,7 +324,13 @@ class Engine final : public EngineBase {
     for (size_t i = 0; i < inst_.size(); i++) {
       InstHost<T, G>& I = inst_[i];
       const size_t gw = (size_t)Q * I.d.n, qw = (size_t)5 * I.L.comp;
-      if ((s = saved.alloc(&gsave[i], gw)) || (s = saved.alloc(&qsave[i], qw))) return s;
+      if ((s = saved.alloc(&gsave[i], gw)) || (s = saved.alloc(&qsave[i], qw))) {
+        const std::string why = err;
+        saved.drop();
+        (void)retry_cells();  // had they made room for the saved state
+        err = why;
+        return s;
+      }
       NLC_CK(cudaMemcpyAsync(gsave[i], I.g[cur0], sizeof(G) * gw, cudaMemcpyDeviceToDevice, st));
       NLC_CK(cudaMemcpyAsync(qsave[i], I.q[cur0].base, sizeof(T) * qw, cudaMemcpyDeviceToDevice,
                              st));
@@ -388,7 +394,7 @@ class Engine final : public EngineBase {
     }
     if ((s = device_error())) return s;
     if ((s = set_chunk(cand[best_k].first, cand[best_k].second))) return s;
-    if ((s = retry_cells())) return s;  // had they made room for the saved state
+    if ((s = retry_cells())) return s;  // as above
     out->best_ms = best;
     out->chunk = 1;
     for (const auto& I : inst_) out->chunk = std::max(out->chunk, I.tz);
@@ -1287,6 +1293,7 @@ class Engine final : public EngineBase {
       I.obs_tiles = list;
       I.obs_part = part;
       I.obs_cap = tl.size();
+      I.obs_tz = 0;  // nothing in it yet
     }
     NLC_CK(cudaMemcpyAsync(I.obs_tiles, tl.data(), sizeof(TileRef) * tl.size(),
                            cudaMemcpyHostToDevice, st));

@@ -236,6 +236,33 @@ def test_autotune_leaves_the_cell_kernels(monkeypatch):
     s.close()
 
 
+def test_autotune_without_room_returns_borrowed_workspaces(monkeypatch):
+    """In a context filled by load_state the saved state may take the room of
+    the cell kernels' workspaces; if it does not fit even so, they come back."""
+    from paper_1907_13415_gb300 import nlc
+    monkeypatch.delenv("NLC_TUNE_CACHE", raising=False)
+    monkeypatch.delenv("NLC_ALLOC_LIMIT", raising=False)
+    w = workload(wl.D3Q19)  # the saved state is the larger of the two here
+    data = initial(w, 0)
+    least = least_limit(lambda: loaded(w, 0, data).close(), monkeypatch)
+    word = 8 * int(np.prod(w.shape))
+    results = set()
+    for words in range(20, 45):
+        monkeypatch.setenv("NLC_ALLOC_LIMIT", str(least + words * word))
+        s = loaded(w, 0, data)
+        first = kernels(s)
+        try:
+            s.autotune(trial_steps=2)
+            tuned = True
+        except nlc.NlcError as e:
+            assert nlc.STATUS[e.status] == "NLC_ENOMEM"
+            tuned = False
+        assert kernels(s) == first
+        results.add((first == CELLS, tuned))
+        s.close()
+    assert {(True, False), (True, True)} <= results
+
+
 def test_missing_mrt_coefficients_and_the_next_fields(monkeypatch):
     """No room for the cell kernels' MRT coefficients: the step takes the
     tiled kernels with that collision; after BGK is back, the next fields

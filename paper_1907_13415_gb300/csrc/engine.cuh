@@ -482,13 +482,11 @@ class Engine final : public EngineBase {
     NLC_CK(cudaMemcpyAsync(&insts_dev_[i].p, &I.p, sizeof(Par<T>), cudaMemcpyHostToDevice,
                            args_.stream));
     if constexpr (kCell) {
-      if (cells_dev_ && !cells_stale_)
-        for (int k = 0; k < 2; k++) {
-          const CellPar c = make_cell_par<Lat>(I.p, k != 0);
-          NLC_CK(cudaMemcpyAsync(&cells_dev_[k * inst_.size() + i].c, &c, sizeof(c),
-                                 cudaMemcpyHostToDevice, args_.stream));
-          NLC_CK(cudaStreamSynchronize(args_.stream));
-        }
+      if (cells_dev_ && !cells_stale_) {
+        const CellPar c[2] = {make_cell_par<Lat>(I.p, false), make_cell_par<Lat>(I.p, true)};
+        NLC_CK(cudaMemcpyAsync(cells_dev_[i].c, c, sizeof(c), cudaMemcpyHostToDevice,
+                               args_.stream));
+      }
     }
     NLC_CK(cudaStreamSynchronize(args_.stream));
     return NLC_OK;
@@ -1174,9 +1172,9 @@ class Engine final : public EngineBase {
         made->push_back(&I);
       }
       const bool fresh = !cells_dev_;
-      if (fresh && (s = alloc(&cells_dev_, 2 * n))) return s;
+      if (fresh && (s = alloc(&cells_dev_, n))) return s;
       if (any_mrt_ && !cell_mrt_ && (s = alloc(&cell_mrt_, n * Q))) return s;
-      std::vector<CellInst<G>> ci(2 * n);
+      std::vector<CellInst<G>> ci(n);
       std::vector<double> rates(n * Q, 0.0);
       int64_t nb = 0;
       for (size_t i = 0; i < n; i++) {
@@ -1184,7 +1182,8 @@ class Engine final : public EngineBase {
         CellInst<G>& C = ci[i];
         C.d = I.d;
         C.L = I.L;
-        C.c = make_cell_par<Lat>(I.p, false);
+        C.c[0] = make_cell_par<Lat>(I.p, false);
+        C.c[1] = make_cell_par<Lat>(I.p, true);
         for (int b = 0; b < 2; b++) {
           C.g[b] = I.g[b];
           C.q[b] = I.q[b].base;
@@ -1198,15 +1197,13 @@ class Engine final : public EngineBase {
           rates[i * Q + k] = mrt_group_coef<Lat, double>(I.rates[k], k);
         C.block0 = (unsigned)nb;
         nb += (I.d.n + CELL_T - 1) / CELL_T;
-        ci[n + i] = C;
-        ci[n + i].c = make_cell_par<Lat>(I.p, true);
       }
       cell_blocks_ = (unsigned)nb;
       cudaStream_t st = args_.stream;
       if (any_mrt_)
         NLC_CK(cudaMemcpyAsync(cell_mrt_, rates.data(), sizeof(double) * n * Q,
                                cudaMemcpyHostToDevice, st));
-      NLC_CK(cudaMemcpyAsync(cells_dev_, ci.data(), sizeof(CellInst<G>) * 2 * n,
+      NLC_CK(cudaMemcpyAsync(cells_dev_, ci.data(), sizeof(CellInst<G>) * n,
                              cudaMemcpyHostToDevice, st));
       NLC_CK(cudaStreamSynchronize(st));
       cells_stale_ = false;
@@ -1221,8 +1218,8 @@ class Engine final : public EngineBase {
       int e[5];
       auto at = [&](int k) { e[k] = mark(); };
       const cudaError_t r =
-          iso_ ? launch_cell_step<Lat, G, true>(cells_dev_ + inst_.size(), (int)inst_.size(),
-                                                cell_blocks_, cur_, any_mrt_, st, at)
+          iso_ ? launch_cell_step<Lat, G, true>(cells_dev_, (int)inst_.size(), cell_blocks_, cur_,
+                                                any_mrt_, st, at)
                : launch_cell_step<Lat, G, false>(cells_dev_, (int)inst_.size(), cell_blocks_,
                                                  cur_, any_mrt_, st, at);
       if (r != cudaSuccess) {
@@ -1715,8 +1712,7 @@ class Engine final : public EngineBase {
   double* hwords_ = nullptr;  // host_words
   size_t hwords_n_ = 0;
   bool hwords_locked_ = false;
-  // float64 arithmetic: descriptors of the cell kernels (ensure_cells), of
-  // every lattice with the standard, then with the isotropic stencils
+  // float64 arithmetic: descriptors of the cell kernels (ensure_cells)
   CellInst<G>* cells_dev_ = nullptr;
   double* cell_mrt_ = nullptr;   // [lattices][Q]
   unsigned cell_blocks_ = 0;

@@ -96,7 +96,7 @@ template <class G>
 struct CellInst {
   Dims d;
   Layout L;
-  CellPar c;
+  CellPar c[2];   // with the standard and the isotropic stencils
   G* g[2];
   double* q[2];   // padded Q, ping-pong
   double* u;      // padded u^n
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(CELL_T) k_cell_stress(const CellInst<G>* __res
   int64_t idx;
   int x, y, z;
   if (!cell_decode(insts, ninst, I, idx, x, y, z)) return;
-  const CellPar c = I->c;
+  const CellPar c = I->c[ISO];
   const Field<double> Q{I->q[cur], I->L};
   const double* p = Q.base + Q.off(0, x, y, z);
   double q[5], d[3][5], s[5], h[5], P[3][3];
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(CELL_T) k_cell_lb(const CellInst<G>* __restric
   int64_t idx;
   int x, y, z;
   if (!cell_decode(insts, ninst, I, idx, x, y, z)) return;
-  const CellPar c = I->c;
+  const CellPar c = I->c[ISO];
   const Dims d = I->d;
   // periodic neighbours: source offsets along each axis, index c + 1
   const int64_t nx = d.nx, nxy = nx * d.ny;
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(CELL_T) k_cell_predict(const CellInst<G>* __re
   int64_t idx;
   int x, y, z;
   if (!cell_decode(insts, ninst, I, idx, x, y, z)) return;
-  const CellPar c = I->c;
+  const CellPar c = I->c[ISO];
   const Field<double> Q{I->q[cur], I->L};
   const int64_t o = Q.off(0, x, y, z), n = I->d.n;
   double q[5], d[3][5], s[5], u[3], g[3][3], h[5], qp[5], mid[5];
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(CELL_T) k_cell_correct(const CellInst<G>* __re
   int64_t idx;
   int x, y, z;
   if (!cell_decode(insts, ninst, I, idx, x, y, z)) return;
-  const CellPar c = I->c;
+  const CellPar c = I->c[ISO];
   const Field<double> QP{I->qp, I->L};
   const int64_t o = QP.off(0, x, y, z), n = I->d.n;
   double q[5], d[3][5], s[5], u[3], g[3][3], h[5], base[5], r[5];

@@ -89,7 +89,6 @@ struct InstHost {
   // MRT coefficients on the device, or nullptr (BGK): s_k / |v_k|^2 for the
   // unfused schedule, then mrt_group_coef(s_k, k) for the step kernels
   T* mrt = nullptr;
-  std::vector<double> rates;  // s_k
   // lazily allocated: unfused schedule, read-back staging, checkpoints
   T* pi = nullptr;
   Field<T> qp;
@@ -435,7 +434,6 @@ class Engine final : public EngineBase {
       if (!I.mrt && (s = alloc(&I.mrt, (size_t)2 * Q))) return s;
       constexpr MomentBasis<Lat> B = make_moment_basis<Lat>();
       T a[2 * Q];
-      I.rates.assign(rates, rates + Q);
       for (int k = 0; k < Q; k++) {
         a[k] = (T)(rates[k] / B.n2[k]);
         a[Q + k] = (T)mrt_group_coef<Lat, double>(rates[k], k);
@@ -444,13 +442,16 @@ class Engine final : public EngineBase {
     }
     const T* ptr = rates ? I.mrt + Q : nullptr;
     NLC_CK(cudaMemcpyAsync(&insts_dev_[i].mrt, &ptr, sizeof(ptr), cudaMemcpyHostToDevice, st));
+    if constexpr (kCell) {
+      if (cells_dev_ && !cells_stale_)
+        NLC_CK(cudaMemcpyAsync(&cells_dev_[i].mrt, &ptr, sizeof(ptr), cudaMemcpyHostToDevice, st));
+    }
     NLC_CK(cudaStreamSynchronize(st));
     mrt_on_[i] = rates != nullptr;
-    cells_stale_ = true;
     any_mrt_ = false;
     for (bool b : mrt_on_) any_mrt_ = any_mrt_ || b;
     drop_graphs();
-    return cells_dev_ ? ensure_cells() : NLC_OK;
+    return NLC_OK;
   }
 
   void invalidate_graphs() override { drop_graphs(); }
@@ -1173,9 +1174,7 @@ class Engine final : public EngineBase {
       }
       const bool fresh = !cells_dev_;
       if (fresh && (s = alloc(&cells_dev_, n))) return s;
-      if (any_mrt_ && !cell_mrt_ && (s = alloc(&cell_mrt_, n * Q))) return s;
       std::vector<CellInst<G>> ci(n);
-      std::vector<double> rates(n * Q, 0.0);
       int64_t nb = 0;
       for (size_t i = 0; i < n; i++) {
         InstHost<T, G>& I = inst_[i];
@@ -1192,17 +1191,12 @@ class Engine final : public EngineBase {
         C.pi = I.pi;
         C.h = I.r1;
         C.qp = I.qp.base;
-        C.mrt = mrt_on_[i] ? cell_mrt_ + i * Q : nullptr;
-        for (int k = 0; k < Q && mrt_on_[i]; k++)
-          rates[i * Q + k] = mrt_group_coef<Lat, double>(I.rates[k], k);
+        C.mrt = mrt_on_[i] ? I.mrt + Q : nullptr;
         C.block0 = (unsigned)nb;
         nb += (I.d.n + CELL_T - 1) / CELL_T;
       }
       cell_blocks_ = (unsigned)nb;
       cudaStream_t st = args_.stream;
-      if (any_mrt_)
-        NLC_CK(cudaMemcpyAsync(cell_mrt_, rates.data(), sizeof(double) * n * Q,
-                               cudaMemcpyHostToDevice, st));
       NLC_CK(cudaMemcpyAsync(cells_dev_, ci.data(), sizeof(CellInst<G>) * n,
                              cudaMemcpyHostToDevice, st));
       NLC_CK(cudaStreamSynchronize(st));
@@ -1714,7 +1708,6 @@ class Engine final : public EngineBase {
   bool hwords_locked_ = false;
   // float64 arithmetic: descriptors of the cell kernels (ensure_cells)
   CellInst<G>* cells_dev_ = nullptr;
-  double* cell_mrt_ = nullptr;   // [lattices][Q]
   unsigned cell_blocks_ = 0;
   bool cells_stale_ = true;      // to be uploaded before the next step
   bool cells_off_ = false;       // workspaces do not fit: tiled kernels

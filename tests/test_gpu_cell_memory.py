@@ -263,19 +263,21 @@ def test_autotune_without_room_returns_borrowed_workspaces(monkeypatch):
     assert {(True, False), (True, True)} <= results
 
 
-def test_missing_mrt_coefficients_and_the_next_fields(monkeypatch):
-    """No room for the cell kernels' MRT coefficients: the step takes the
-    tiled kernels with that collision; after BGK is back, the next fields
-    bring the cell kernels back too."""
+def test_mrt_takes_no_more_than_its_coefficients(monkeypatch):
+    """With room for the coefficients the cell kernels go on with MRT, without
+    it the collision is refused and BGK stays."""
+    from paper_1907_13415_gb300 import nlc
     w = workload(wl.D2Q9)
     Q0, r = w.initial_q5(), rates(w)
+    want = {}
     monkeypatch.delenv("NLC_ALLOC_LIMIT", raising=False)
-    ref = make(w, 0)
-    ref.set_fields(Q0)
-    ref.set_mrt(r)
-    ref.step(3)
-    want = ref.get_fields()[0]
-    ref.close()
+    for mrt in (False, True):
+        ref = make(w, 0)
+        ref.set_fields(Q0)
+        ref.set_mrt(r if mrt else None)
+        ref.step(3)
+        want[mrt] = ref.get_fields()[0]
+        ref.close()
 
     def fields():
         s = make(w, 0)
@@ -283,24 +285,22 @@ def test_missing_mrt_coefficients_and_the_next_fields(monkeypatch):
         s.get_fields()
         return s
 
-    # the descriptors of the cell kernels, found in steps of less than their
-    # MRT coefficients (72 bytes), and the coefficients of the tiled ones
     limit = least_limit(lambda: fields().close(), monkeypatch)
-    for limit in range(limit, limit + 4096, 32):
+    for limit in range(limit, limit + 4096, 32):  # and the cell kernels' descriptors
         monkeypatch.setenv("NLC_ALLOC_LIMIT", str(limit))
         s = fields()
         used = kernels(s)
         s.close()
         if used == CELLS:
             break
-    monkeypatch.setenv("NLC_ALLOC_LIMIT", str(limit + 8 * 2 * 9))
-    s = fields()
-    assert kernels(s) == CELLS
-    s.set_fields(Q0)
-    s.set_mrt(r)
-    assert kernels(s, 3) == TILED
-    assert rel(s.get_fields()[0], want) < 1e-12
-    s.set_mrt(None)
-    s.set_fields(Q0)
-    assert kernels(s) == CELLS
-    s.close()
+    for extra, mrt in ((0, False), (8 * 2 * 9, True)):
+        monkeypatch.setenv("NLC_ALLOC_LIMIT", str(limit + extra))
+        s = fields()
+        if mrt:
+            s.set_mrt(r)
+        else:
+            with pytest.raises(nlc.NlcError):
+                s.set_mrt(r)
+        assert kernels(s, 3) == CELLS
+        assert np.array_equal(s.get_fields()[0], want[mrt])
+        s.close()

@@ -1383,21 +1383,25 @@ class Engine final : public EngineBase {
       if ((s = plan_tiled_reverse(I))) return s;
     }
     if (I.seg_grid <= 0 || I.rec_len >= len) return NLC_OK;
-    const int64_t n = I.d.n, comp = I.L.comp;
-    for (int b = 0; b < 2; b++)
-      if ((s = alloc(&I.rec_g[b], (size_t)((len + 1) * Q * n))) ||
-          (s = alloc(&I.rec_q[b], (size_t)((len + 1) * 5 * comp))) ||
-          (s = alloc(&I.rec_pi[b], (size_t)(len * DIM * DIM * n))) ||
-          (s = alloc(&I.rec_u[b], (size_t)(len * DIM * comp))) ||
-          (s = alloc(&I.rec_qp[b], (size_t)(len * 5 * comp))) ||
-          (s = alloc(&I.rec_r1[b], (size_t)(5 * n))))
-        return s;
-    I.rec_len = len;
     if (!side_stream_) {
-      NLC_CK(cudaStreamCreateWithFlags(&side_stream_, cudaStreamNonBlocking));
       for (int k = 0; k < 5; k++)
-        NLC_CK(cudaEventCreateWithFlags(&seg_ev_[k], cudaEventDisableTiming));
+        if (!seg_ev_[k]) NLC_CK(cudaEventCreateWithFlags(&seg_ev_[k], cudaEventDisableTiming));
+      NLC_CK(cudaStreamCreateWithFlags(&side_stream_, cudaStreamNonBlocking));
     }
+    const int64_t n = I.d.n, comp = I.L.comp;
+    const int64_t words[6] = {(len + 1) * Q * n,  (len + 1) * 5 * comp, len * DIM * DIM * n,
+                              len * DIM * comp,   len * 5 * comp,       5 * n};
+    Group mem(*this);
+    T* w[2][6];
+    for (int b = 0; b < 2; b++)
+      for (int k = 0; k < 6; k++)
+        if ((s = mem.alloc(&w[b][k], (size_t)words[k]))) return s;
+    mem.kept = true;
+    for (int b = 0; b < 2; b++) {
+      I.rec_g[b] = w[b][0], I.rec_q[b] = w[b][1], I.rec_pi[b] = w[b][2];
+      I.rec_u[b] = w[b][3], I.rec_qp[b] = w[b][4], I.rec_r1[b] = w[b][5];
+    }
+    I.rec_len = len;
     return NLC_OK;
   }
 

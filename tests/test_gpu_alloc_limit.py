@@ -55,7 +55,9 @@ def calls(sim, w, saved, adjoint):
            ("save", lambda: np.frombuffer(sim.save(), dtype=np.uint8)[64:])]
     if adjoint:
         out += [("set_fields_again", lambda: sim.set_fields(Q0)),
-                ("adjoint", lambda: sim.adjoint(3.0, 1.0, 1.0, 5, 2)["dQ0"])]
+                ("adjoint", lambda: sim.adjoint(3.0, 1.0, 1.0, 5, 2)["dQ0"]),
+                ("set_fields_third", lambda: sim.set_fields(Q0)),
+                ("adjoint_longer", lambda: sim.adjoint(3.0, 1.0, 1.0, 7, 4)["dQ0"])]
     return out
 
 
